@@ -153,7 +153,7 @@ void d2moe_carve_workspace(const d2moe_config* c, long long T, Workspace* ws) {
     ws->off_status = take(256);
     ws->off_logits = take((size_t)T * c->n_experts * 4);
     ws->off_keys = take(A * 4);
-    ws->off_hist = take(n_keys * 4);
+    ws->off_hist = take(D2MOE_HIST_RUNS * n_keys * 4);
     ws->off_topk_idx = take(A * 4);
     ws->off_topk_w = take(A * 4);
     ws->off_bit_idx = take(A);
@@ -245,7 +245,7 @@ extern "C" d2moe_status d2moe_route(const d2moe_config* c, int64_t T, const void
     launch_chain_begin();
     cudaError_t e = launch_route(D, (const __nv_bfloat16*)x, (const __nv_bfloat16*)gate_w, logits,
                                  (const __nv_bfloat16*)bit_w, forced, R, (float*)(w + ws.off_logits),
-                                 (int32_t*)(w + ws.off_keys), (int32_t*)(w + ws.off_hist), device_status, st);
+                                 (int32_t*)(w + ws.off_keys), (int32_t*)(w + ws.off_hist), (int)(D2MOE_HIST_RUNS * n_keys), device_status, st);
     return e == cudaSuccess ? D2MOE_OK : D2MOE_ERR_CUDA;
 }
 
@@ -313,7 +313,7 @@ static d2moe_status forward_impl(const d2moe_config* c, int64_t T, const void* x
         e = launch_route(D, (const __nv_bfloat16*)x, (const __nv_bfloat16*)in->gate_w_bf16, in->logits,
                          (const __nv_bfloat16*)in->bit_w_bf16, in->forced_bit_idx, R,
                          (float*)(w + ws.off_logits), (int32_t*)(w + ws.off_keys),
-                         (int32_t*)(w + ws.off_hist), device_status, st, want_defer ? &group_deferred : nullptr);
+                         (int32_t*)(w + ws.off_hist), (int)(D2MOE_HIST_RUNS * D.E * D.K), device_status, st, want_defer ? &group_deferred : nullptr);
         if (e != cudaSuccess) return D2MOE_ERR_CUDA;
     }
     ExpertPtrs P;
@@ -335,7 +335,7 @@ static d2moe_status forward_impl(const d2moe_config* c, int64_t T, const void* x
         B.slot_f = (float*)(w + ws.off_slot_f);
         e = pl.decode ? launch_ffn_i8(c, D, Lgu, Ld, P, (const __nv_bfloat16*)x, R, pl, B, device_status, st, ev,
                                       group_deferred ? (const int32_t*)(w + ws.off_keys) : nullptr)
-                      : launch_ffn_tensor(c, D, Lgu, Ld, P, (const __nv_bfloat16*)x, R, pl, B, device_status, st, ev);
+                      : launch_ffn_tensor(c, D, Lgu, Ld, P, (const __nv_bfloat16*)x, R, pl, B, device_status, st, ev, pre != nullptr);
         if (e != cudaSuccess) return D2MOE_ERR_CUDA;
         mark(3);
         e = launch_combine(D, R, B.o32, pl.n_split, (size_t)pl.R_alloc * D.d, B.row_map,
@@ -386,18 +386,18 @@ extern "C" d2moe_status d2moe_selftest_wait_expiry(int which, int32_t* device_st
 
 extern "C" int d2moe_forward_launch_count(const d2moe_config* c, int64_t T, int routing_precomputed) {
     if (d2moe_check_config(c) != D2MOE_OK || T <= 0) return 0;
-    // route, then count + scan + scatter (one launch when the load is small: the rule of launch_route)
+    // route, then the grouping (two launches for a large load, one otherwise: the rule of launch_route)
     const long long A = (long long)T * c->top_k, n_keys = (long long)c->n_experts * c->n_bits;
     const bool small = A <= 8192 && n_keys <= 2048 && n_keys * ((A + 31) / 32) <= 1024;
-    int route = routing_precomputed ? 0 : (small || d2moe_group_is_sortable(A, n_keys) || d2moe_group_is_mid(A, n_keys) ? 2 : 4);
+    int route = routing_precomputed ? 0 : (small || d2moe_group_is_sortable(A, n_keys) || d2moe_group_is_mid(A, n_keys) ? 2 : 3);
     if (!routing_precomputed && (small || d2moe_group_is_sortable(A, n_keys)) && use_tensor_path(c)) {   // grouping inside the decode path's unit build
         TcPlan pl0;
         tc_plan(c, T, &pl0);
         if (pl0.decode) route -= 1;
     }
-    // more than 16 experts: the gate logits come from a tiled kernel of their own (when the caller supplies
+    // more than 16 experts or many tokens: the gate logits come from a tiled kernel of their own (when the caller supplies
     // logits instead of gate weights that launch does not happen: the count is then one too high)
-    if (!routing_precomputed && c->n_experts > 16 && (size_t)c->d_model * 2 * 16 <= 200 * 1024) route += 1;
+    if (!routing_precomputed && (c->n_experts > 16 || T >= 256) && (size_t)c->d_model * 2 * 2 <= 190 * 1024) route += 1;
     if (use_tensor_path(c)) {
         TcPlan pl;
         tc_plan(c, T, &pl);

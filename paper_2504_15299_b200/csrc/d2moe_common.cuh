@@ -195,10 +195,12 @@ struct RouteBufs {
 // Grouping of the assignments by (expert, width) key: the single-block kernel takes the smallest loads (its
 // rule is in launch_route), a single-block counting sort loads of up to 4096 assignments on up to 512 keys, one
 // launch of a few blocks the other mid-sized ones (every block counts all keys: the walks per warp must stay
-// short), histogram + scan + scatter kernels the rest.  All give the same (unique) stable order.
+// short), a counting sort over the grid (two launches) the rest.  All give the same (unique) stable order.
 static inline bool d2moe_group_is_mid(long long A, long long n_keys) {
     return A <= 12288 && n_keys <= 2048 && n_keys * ((A + 31) / 32) <= 6144;
 }
+
+constexpr size_t D2MOE_HIST_RUNS = 64;     // histograms the workspace holds for the grouping of large loads
 
 // Workspace carving (all offsets 256-byte aligned).
 struct Workspace {
@@ -224,7 +226,7 @@ cudaError_t launch_unpack_scales(const PackLayout& L, const uint8_t* packed, flo
 // kernels_route.cu
 cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bfloat16* gate_w,
                          const float* logits_in, const __nv_bfloat16* bit_w, const int8_t* forced,
-                         const RouteBufs& R, float* logits_ws, int32_t* keys_ws, int32_t* hist_ws,
+                         const RouteBufs& R, float* logits_ws, int32_t* keys_ws, int32_t* hist_ws, int hist_ints,
                          int32_t* device_status, cudaStream_t st, bool* defer_small_group = nullptr);
 // the single-block grouping rule of launch_route (decode-sized loads)
 static inline bool d2moe_group_is_small(long long A, long long n_keys) {

@@ -171,19 +171,36 @@ __global__ void combine4_kernel(MoeDims D, RouteBufs R, const float* __restrict_
         acc[0] = __low2float(r01); acc[1] = __high2float(r01); acc[2] = __low2float(r23); acc[3] = __high2float(r23);
     }
     float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int s = 0; s < D.k + D.n_shared; ++s) {
-        const int a = s < D.k ? t * D.k + s : D.A + (s - D.k) * D.T + t;
-        const float w = s < D.k ? R.topk_w[a] : 1.0f;
-        const long long rowi = row_map ? (long long)row_map[a] : (long long)a;
-        if (rowi < 0) continue;                      // an assignment that was skipped (bad routing index)
-        const size_t row = (size_t)rowi;
-        float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        for (int sp = 0; sp < n_split; ++sp) {
-            const float4 v = *reinterpret_cast<const float4*>(obuf + sp * split_stride + row * D.d + c);
-            o[0] += v.x; o[1] += v.y; o[2] += v.z; o[3] += v.w;
-        }
+    // four partial rows (slot by slot, split by split) at a time: their row numbers and weights first, then all their loads, so
+    // that a token waits for two trips to memory per four rows, not per row
+    const int n = (D.k + D.n_shared) * n_split;
+    float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int q0 = 0; q0 < n; q0 += 4) {
+        long long row[4];
+        float w[4];
+        int sp[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) sum[i] = fmaf(w, o[i], sum[i]);
+        for (int j = 0; j < 4; ++j) {
+            const int q = min(q0 + j, n - 1), s = q / n_split;
+            const int a = s < D.k ? t * D.k + s : D.A + (s - D.k) * D.T + t;
+            sp[j] = q0 + j < n ? q - s * n_split : -1;
+            row[j] = row_map ? (long long)row_map[a] : (long long)a;           // -1: skipped (bad routing index)
+            w[j] = s < D.k ? R.topk_w[a] : 1.0f;
+        }
+        float4 v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (row[j] >= 0 && sp[j] >= 0) v[j] = *reinterpret_cast<const float4*>(obuf + sp[j] * split_stride + (size_t)row[j] * D.d + c);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (row[j] < 0 || sp[j] < 0) continue;
+            if (sp[j] == 0) { o[0] = v[j].x; o[1] = v[j].y; o[2] = v[j].z; o[3] = v[j].w; }
+            else { o[0] += v[j].x; o[1] += v[j].y; o[2] += v[j].z; o[3] += v[j].w; }
+            if (sp[j] == n_split - 1) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) sum[i] = fmaf(w[j], o[i], sum[i]);
+            }
+        }
     }
     __nv_bfloat162 y01, y23;
     y01.x = __float2bfloat16_rn(acc[0] + sum[0]); y01.y = __float2bfloat16_rn(acc[1] + sum[1]);
@@ -196,26 +213,65 @@ __global__ void combine4_kernel(MoeDims D, RouteBufs R, const float* __restrict_
 
 // xn = bf16( x / sqrt(mean(x^2) + eps) ), fp64 inside so the rounding matches a double-precision
 // evaluation; one block per token.
-__global__ void __launch_bounds__(256)
-rmsnorm_kernel(int d, double eps, const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ xn) {
+// (A row of up to 8192 elements is read once, 16 bytes per load, and kept in registers between the sum and the scaling; 16
+// tokens of 4096: 11 us before, with 2-byte loads and the row read twice.)
+__global__ void __launch_bounds__(512)
+rmsnorm_kernel(int d, double eps, const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ xn, int vec) {
     pdl_enter();
-    __shared__ double red[8];
-    const int t = blockIdx.x;
+    __shared__ double red[16];
+    const int t = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const __nv_bfloat16* xt = x + (size_t)t * d;
+    __nv_bfloat16* yt = xn + (size_t)t * d;
+    auto total = [&](double ss) {
+        for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+        if (lane == 0) red[warp] = ss;
+        __syncthreads();
+        double tot = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
+        return 1.0 / sqrt(tot / (double)d + eps);
+    };
+    if (vec) {                                    // d <= 16 blockDim.x, rows 16-byte aligned, d a multiple of 8
+        uint4 raw[2];
+        double s4[4] = {0.0, 0.0, 0.0, 0.0};      // short chains: fp64 additions are slow
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = threadIdx.x + k * blockDim.x;
+            raw[k] = i < d / 8 ? reinterpret_cast<const uint4*>(xt)[i] : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t w4[4] = {raw[k].x, raw[k].y, raw[k].z, raw[k].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float a = __uint_as_float(w4[j] << 16), b = __uint_as_float(w4[j] & 0xffff0000u);
+                s4[j] += (double)a * a + (double)b * b;
+            }
+        }
+        const double inv = total((s4[0] + s4[1]) + (s4[2] + s4[3]));
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = threadIdx.x + k * blockDim.x;
+            if (i >= d / 8) continue;
+            const uint32_t w4[4] = {raw[k].x, raw[k].y, raw[k].z, raw[k].w};
+            uint32_t o4[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                __nv_bfloat162 o;
+                o.x = __float2bfloat16_rn((float)((double)__uint_as_float(w4[j] << 16) * inv));
+                o.y = __float2bfloat16_rn((float)((double)__uint_as_float(w4[j] & 0xffff0000u) * inv));
+                o4[j] = *reinterpret_cast<uint32_t*>(&o);
+            }
+            reinterpret_cast<uint4*>(yt)[i] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+        }
+        return;
+    }
     double ss = 0.0;
     for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        const double v = (double)__bfloat162float(x[(size_t)t * d + i]);
+        const double v = (double)__bfloat162float(xt[i]);
         ss += v * v;
     }
-    for (int off = 16; off; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    double tot = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-    const double inv = 1.0 / sqrt(tot / (double)d + eps);
-    for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        const double v = (double)__bfloat162float(x[(size_t)t * d + i]) * inv;
-        xn[(size_t)t * d + i] = __float2bfloat16_rn((float)v);
-    }
+    const double inv = total(ss);
+    for (int i = threadIdx.x; i < d; i += blockDim.x) yt[i] = __float2bfloat16_rn((float)((double)__bfloat162float(xt[i]) * inv));
 }
 
 }  // namespace
@@ -256,6 +312,7 @@ cudaError_t launch_combine(const MoeDims& D, const RouteBufs& R, const float* ob
 
 cudaError_t launch_rmsnorm(int T, int d, float eps, const __nv_bfloat16* x, __nv_bfloat16* xn, cudaStream_t st) {
     if (T == 0) return cudaSuccess;
-    launch_chained(rmsnorm_kernel, dim3(T), dim3(256), 0, st, d, (double)eps, x, xn);
+    const int vec = d <= 8192 && d % 8 == 0 && (((uintptr_t)x | (uintptr_t)xn) & 15) == 0;
+    launch_chained(rmsnorm_kernel, dim3(T), dim3(512), 0, st, d, (double)eps, x, xn, vec);
     return cudaGetLastError();
 }

@@ -136,61 +136,83 @@ route_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16
     }
 }
 
-// One warp per key: count the assignments that carry it.
-__global__ void count_kernel(int A, int n_keys, const int32_t* __restrict__ keys, int32_t* __restrict__ hist) {
+// Grouping of large loads: a stable counting sort over the grid.  Block b owns a contiguous run of assignments and takes it 32
+// per warp at a time; an assignment's rank among the earlier ones of its key inside the run comes from a match instruction and
+// running counts in shared memory (per warp, then summed over warps: warps own contiguous pieces of each 1024).  Pass 1 leaves
+// the ranks in inv_perm and the run's histogram in hist[b]; pass 2 adds the counts of the earlier runs and of the smaller keys.
+// (Before: one warp per key walked all assignments, twice: 62 us for 9000 assignments on 192 keys.)
+constexpr int GS_THREADS = 512, GS_MAX_RUNS = 64;
+__global__ void __launch_bounds__(GS_THREADS)
+run_rank_kernel(int A, int n_keys, int run, const int32_t* __restrict__ keys, int32_t* __restrict__ rank, int32_t* __restrict__ hist) {
     pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const int key = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (key >= n_keys) return;
-    int cnt = 0;
-    for (int base = 0; base < A; base += 32) {
-        const int a = base + lane;
-        const bool m = a < A && keys[a] == key;
-        cnt += __popc(__ballot_sync(0xffffffffu, m));
+    extern __shared__ int32_t s_run[];            // [n_keys] counts of the run so far, then one warp's turn at a time
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < n_keys; i += GS_THREADS) s_run[i] = 0;
+    __syncthreads();
+    const int a0 = blockIdx.x * run, a1 = min(A, a0 + run);
+    for (int base = a0; base < a1; base += GS_THREADS) {
+        const int a = base + threadIdx.x;
+        const int key = a < a1 ? keys[a] : -1 - lane;                  // dead lanes match nobody
+        const unsigned same = __match_any_sync(0xffffffffu, key);
+        const int mine = __popc(same & ((1u << lane) - 1u));
+        // the warps add their counts in order (stable): sixteen short turns per 512 assignments
+        int before = 0;
+        for (int w = 0; w < GS_THREADS / 32; ++w) {
+            if (w == warp) {
+                if (a < a1) before = s_run[key];
+                __syncwarp();
+                if (a < a1 && mine == 0) s_run[key] = before + __popc(same);
+            }
+            __syncthreads();
+        }
+        if (a < a1) rank[a] = before + mine;
     }
-    if (lane == 0) hist[key] = cnt;
+    for (int i = threadIdx.x; i < n_keys; i += GS_THREADS) hist[(size_t)blockIdx.x * n_keys + i] = s_run[i];
 }
 
-// Exclusive prefix sum of the histogram by one warp.
-__global__ void scan_kernel(int n_keys, const int32_t* __restrict__ hist, int32_t* __restrict__ group_off) {
+__global__ void __launch_bounds__(GS_THREADS)
+run_place_kernel(int A, int n_keys, int run, int n_runs, const int32_t* __restrict__ keys, const int32_t* __restrict__ hist,
+                 int32_t* __restrict__ group_off, int32_t* __restrict__ perm, int32_t* inv_perm) {
     pdl_enter();
-    const int lane = threadIdx.x;
-    int carry = 0;
-    for (int base = 0; base < n_keys; base += 32) {
-        const int i = base + lane;
-        const int v = i < n_keys ? hist[i] : 0;
-        int incl = v;
+    extern __shared__ int32_t s_place[];          // [n_keys] first position of this run's assignments of a key
+    __shared__ int s_warp[GS_THREADS / 32];
+    __shared__ int s_carry;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_carry = 0;
+    __syncthreads();
+    for (int k0 = 0; k0 < n_keys; k0 += GS_THREADS) {
+        const int key = k0 + threadIdx.x;
+        int total = 0, earlier = 0;
+        if (key < n_keys)
+            for (int r = 0; r < n_runs; ++r) {
+                const int c = hist[(size_t)r * n_keys + key];
+                if (r == (int)blockIdx.x) earlier = total;
+                total += c;
+            }
+        int incl = total;                         // block-wide exclusive scan of the keys' totals
         for (int off = 1; off < 32; off <<= 1) {
             const int o = __shfl_up_sync(0xffffffffu, incl, off);
             if (lane >= off) incl += o;
         }
-        if (i < n_keys) group_off[i] = carry + incl - v;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) group_off[n_keys] = carry;
-}
-
-// One warp per key: write its assignments, in ascending assignment id, from group_off[key] on.
-__global__ void scatter_kernel(int A, int n_keys, const int32_t* __restrict__ keys,
-                               const int32_t* __restrict__ group_off, int32_t* __restrict__ perm,
-                               int32_t* __restrict__ inv_perm) {
-    pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const int key = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (key >= n_keys) return;
-    int pos = group_off[key];
-    const int end = group_off[key + 1];
-    if (pos == end) return;
-    for (int base = 0; base < A; base += 32) {
-        const int a = base + lane;
-        const bool m = a < A && keys[a] == key;
-        const unsigned bal = __ballot_sync(0xffffffffu, m);
-        if (m) {
-            const int p = pos + __popc(bal & ((1u << lane) - 1u));
-            perm[p] = a;
-            inv_perm[a] = p;
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        int carry = s_carry;
+        for (int w = 0; w < warp; ++w) carry += s_warp[w];
+        const int off = carry + incl - total;
+        if (key < n_keys) {
+            s_place[key] = off + earlier;
+            if (blockIdx.x == 0) group_off[key] = off;
         }
-        pos += __popc(bal);
+        __syncthreads();
+        if (threadIdx.x == GS_THREADS - 1) s_carry = carry + incl;
+        __syncthreads();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) group_off[n_keys] = A;
+    const int a0 = blockIdx.x * run, a1 = min(A, a0 + run);
+    for (int a = a0 + threadIdx.x; a < a1; a += GS_THREADS) {
+        const int p = s_place[keys[a]] + inv_perm[a];
+        perm[p] = a;
+        inv_perm[a] = p;
     }
 }
 
@@ -237,27 +259,109 @@ __device__ __forceinline__ void stage_row(__nv_bfloat16* dst, const __nv_bfloat1
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Gate logits for many experts: a block stages TB token rows and EB weight rows once and forms the
-// TB x EB dot products (pinned order), so a weight row is read once per TB tokens instead of per token.
-__global__ void __launch_bounds__(256)
-gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
-                   float* __restrict__ logits, int TB, int EB) {
-    pdl_enter();
-    extern __shared__ __align__(16) uint8_t rsm[];
-    __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(rsm);
-    __nv_bfloat16* ws = xs + (size_t)TB * d;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t0 = blockIdx.x * TB, e0 = blockIdx.y * EB;
-    const int nt = min(TB, T - t0), ne = min(EB, E - e0);
-    stage_row(xs, x + (size_t)t0 * d, nt * d);                 // consecutive rows are contiguous: one copy loop each
-    stage_row(ws, gate_w + (size_t)e0 * d, ne * d);
-    stage_wait();
-    __syncthreads();
-    for (int pr = warp; pr < nt * ne; pr += 8) {
-        const int tt = pr / ne, ee = pr - tt * ne;
-        const float v = dot_pinned_smem(xs + (size_t)tt * d, ws + (size_t)ee * d, d, lane);
-        if (lane == 0) logits[(size_t)(t0 + tt) * E + e0 + ee] = v;
+// Dot products of one row with NR others, all in shared memory, by 16 lanes: lane p of the half-warp carries the chains 2p and
+// 2p + 1 of the pinned order (elements 2p, 2p + 1 of every 32), so an operand is one 4-byte load per 32 elements and the
+// row's word is used NR times.  Afterwards the butterfly: chain distance 16, 8, 4, 2 is lane distance 8, 4, 2, 1;
+// distance 1 is the lane's own pair.  d a multiple of 32.
+template <int NR>
+__device__ __forceinline__ void dots_halfwarp(const uint32_t* x, const uint32_t* const (&wr)[NR], int d, float (&out)[NR]) {
+    const int p = threadIdx.x & 15;
+    float acc[NR][2];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc[r][0] = acc[r][1] = 0.0f;
+#pragma unroll 8
+    for (int i = 0; i < d / 32; ++i) {
+        const uint32_t xw = x[16 * i + p];
+        const float x0 = __uint_as_float(xw << 16), x1 = __uint_as_float(xw & 0xffff0000u);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const uint32_t v = wr[r][16 * i + p];
+            acc[r][0] = fmaf(x0, __uint_as_float(v << 16), acc[r][0]);
+            acc[r][1] = fmaf(x1, __uint_as_float(v & 0xffff0000u), acc[r][1]);
+        }
     }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+#pragma unroll
+        for (int off = 8; off; off >>= 1) {
+            acc[r][0] += __shfl_xor_sync(0xffffffffu, acc[r][0], off);
+            acc[r][1] += __shfl_xor_sync(0xffffffffu, acc[r][1], off);
+        }
+        out[r] = acc[r][0] + acc[r][1];
+    }
+}
+
+// Gate logits as a tiled product: a block takes 16 tokens x 8 experts, a half-warp forms 4 x 4 of them in registers (same lane
+// layout and order as above), columns stream through shared memory 256 at a time, three stages deep.  Bound: fp32 issue (a
+// multiply-add, half a conversion and a quarter of a shared load per product).
+// 1500 tokens x 64 experts x 2048: 62 us before (one dot per warp, two 2-byte shared loads per product).
+constexpr int GATE_TB = 16, GATE_EB = 8, GATE_COLS = 256, GATE_STAGES = 3;
+constexpr int GATE_PITCH = GATE_COLS / 2 + 4;           // words per row: four rows on, the other half of the banks
+__global__ void __launch_bounds__(128)
+gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
+                   float* __restrict__ logits) {
+    pdl_enter();
+    constexpr int ROWS = GATE_TB + GATE_EB;
+    __shared__ __align__(16) uint32_t sm[GATE_STAGES][ROWS][GATE_PITCH];
+    const int hw = threadIdx.x >> 4, p = threadIdx.x & 15;
+    const int tb = blockIdx.x * GATE_TB, eb = blockIdx.y * GATE_EB;
+    const int n_chunks = (d + GATE_COLS - 1) / GATE_COLS;
+    auto stage = [&](int c) {
+        if (c < n_chunks) {
+            const int c0 = c * GATE_COLS, n16 = min(GATE_COLS, d - c0) / 8;
+            for (int i = threadIdx.x; i < ROWS * (GATE_COLS / 8); i += 128) {
+                const int r = i / (GATE_COLS / 8), k = i % (GATE_COLS / 8);
+                if (k >= n16) continue;
+                // rows past the end repeat the last one; their results are dropped
+                const __nv_bfloat16* src = r < GATE_TB ? x + (size_t)min(tb + r, T - 1) * d : gate_w + (size_t)min(eb + r - GATE_TB, E - 1) * d;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(&sm[c % GATE_STAGES][r][4 * k])), "l"(src + c0 + 8 * k) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < GATE_STAGES - 1; ++c) stage(c);
+    float acc[4][4][2];
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[t][r][0] = acc[t][r][1] = 0.0f;
+    const int xr = (hw & 3) * 4, wr = GATE_TB + (hw >> 2) * 4;
+    for (int c = 0; c < n_chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(GATE_STAGES - 2) : "memory");
+        __syncthreads();                          // chunk c is there; the stage refilled next has been read
+        stage(c + GATE_STAGES - 1);
+        const uint32_t (*b)[GATE_PITCH] = sm[c % GATE_STAGES];
+        const int steps = min(GATE_COLS, d - c * GATE_COLS) / 32;
+#pragma unroll 4
+        for (int i = 0; i < steps; ++i) {
+            float xv[4][2], wv[4][2];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const uint32_t v = b[xr + t][16 * i + p], u = b[wr + t][16 * i + p];
+                xv[t][0] = __uint_as_float(v << 16); xv[t][1] = __uint_as_float(v & 0xffff0000u);
+                wv[t][0] = __uint_as_float(u << 16); wv[t][1] = __uint_as_float(u & 0xffff0000u);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    acc[t][r][0] = fmaf(xv[t][0], wv[r][0], acc[t][r][0]);
+                    acc[t][r][1] = fmaf(xv[t][1], wv[r][1], acc[t][r][1]);
+                }
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+#pragma unroll
+            for (int off = 8; off; off >>= 1) {
+                acc[t][r][0] += __shfl_xor_sync(0xffffffffu, acc[t][r][0], off);
+                acc[t][r][1] += __shfl_xor_sync(0xffffffffu, acc[t][r][1], off);
+            }
+            const int tt = tb + xr + t, ee = eb + wr - GATE_TB + r;
+            if (p == 4 * t + r && tt < T && ee < E) logits[(size_t)tt * E + ee] = acc[t][r][0] + acc[t][r][1];
+        }
 }
 
 // One block (8 warps) per token: the same results as route_kernel, with the token row and batches of
@@ -267,19 +371,20 @@ __global__ void __launch_bounds__(256)
 route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
                    const float* __restrict__ logits_in, const __nv_bfloat16* __restrict__ bit_w,
                    const int8_t* __restrict__ forced, RouteBufs R, int32_t* __restrict__ keys,
-                   int32_t* __restrict__ device_status, int EB) {
+                   int32_t* __restrict__ device_status, int EB, int ws_elems, int slot_pitch) {
     pdl_enter();
     extern __shared__ __align__(16) uint8_t rsm[];
+    // EB == 0: nothing is staged (logits and widths supplied); ws_elems: elements of the staging area behind the token row
     __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(rsm);
-    __nv_bfloat16* ws = xs + D.d;
-    float* lg_s = reinterpret_cast<float*>(ws + (size_t)EB * D.d);     // [E]
+    __nv_bfloat16* ws = xs + (EB ? D.d : 0);
+    float* lg_s = reinterpret_cast<float*>(ws + ws_elems);               // [E]
     float* u_s = lg_s + D.E;                                             // [k * K]
     int* sel_s = reinterpret_cast<int*>(u_s + MAX_TOPK * 8);             // [k]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = blockIdx.x;
     const int E = D.E;
 
-    if (!(logits_in && forced)) stage_row(xs, x + (size_t)t * D.d, D.d);
+    if (EB) stage_row(xs, x + (size_t)t * D.d, D.d);
     if (logits_in) {
         for (int e = threadIdx.x; e < E; e += blockDim.x) lg_s[e] = logits_in[(size_t)t * E + e];
         stage_wait();
@@ -317,7 +422,36 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
     }
     __syncthreads();
 
-    if (!forced) {              // bit-width router logits of the selected experts: rows (slot s, width c)
+    if (!forced && slot_pitch) {       // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
+        for (int s = 0; s < D.k; ++s)         // (odd slots half a bank row on: the two half-warps of a warp meet no conflict)
+            stage_row(ws + (size_t)s * slot_pitch, bit_w + (size_t)sel_s[s] * D.K * D.d, D.K * D.d);
+        stage_wait();
+        __syncthreads();
+        if (D.k * D.K <= (int)(blockDim.x >> 4)) {                             // few rows: a half-warp each (shortest chain)
+            const int row = min((int)(threadIdx.x >> 4), D.k * D.K - 1), s = row / D.K, c = row - s * D.K;
+            const uint32_t* wr[1] = {reinterpret_cast<const uint32_t*>(ws + (size_t)s * slot_pitch + (size_t)c * D.d)};
+            float v[1];
+            dots_halfwarp<1>(reinterpret_cast<const uint32_t*>(xs), wr, D.d, v);
+            if ((threadIdx.x & 15) == 0 && (int)(threadIdx.x >> 4) < D.k * D.K) u_s[row] = v[0];
+        } else
+        for (int sb = 0; sb < D.k; sb += (int)(blockDim.x >> 4)) {
+            const int s = min(sb + (int)(threadIdx.x >> 4), D.k - 1);
+            if (sb + (int)(threadIdx.x >> 5) * 2 >= D.k) break;               // nothing for this warp
+            for (int c0 = 0; c0 < D.K; c0 += 4) {
+                const uint32_t* wr[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)       // past the end: the last row again, result dropped
+                    wr[r] = reinterpret_cast<const uint32_t*>(ws + (size_t)s * slot_pitch + (size_t)min(c0 + r, D.K - 1) * D.d);
+                float v[4];
+                dots_halfwarp<4>(reinterpret_cast<const uint32_t*>(xs), wr, D.d, v);
+                const int p = threadIdx.x & 15;
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (p == r && c0 + r < D.K) u_s[s * D.K + c0 + r] = v[r];
+            }
+        }
+        __syncthreads();
+    } else if (!forced) {       // bit-width router logits of the selected experts: rows (slot s, width c)
         const int n_rows = D.k * D.K;
         for (int rb = 0; rb < n_rows; rb += EB) {
             const int n = min(EB, n_rows - rb);
@@ -365,7 +499,7 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
 
 cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bfloat16* gate_w,
                          const float* logits_in, const __nv_bfloat16* bit_w, const int8_t* forced,
-                         const RouteBufs& R, float* logits_ws, int32_t* keys_ws, int32_t* hist_ws,
+                         const RouteBufs& R, float* logits_ws, int32_t* keys_ws, int32_t* hist_ws, int hist_ints,
                          int32_t* device_status, cudaStream_t st, bool* defer_small_group) {
     const int warps_per_block = 4;
     const int n_keys = D.E * D.K;
@@ -376,23 +510,29 @@ cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bf
     int EB = row_bytes + tail_bytes < budget ? (int)((budget - row_bytes - tail_bytes) / row_bytes) : 0;
     if (EB > 8) EB = 8;
     if (EB >= 1 && D.d % 8 == 0) {
-        // many experts: gate logits by the tiled kernel first, then route from those logits
-        if (!logits_in && D.E > 16 && logits_ws && 16 * row_bytes <= budget) {
-            const int TB = 8, EBL = 8;
-            const size_t lsm = (size_t)(TB + EBL) * row_bytes;
-            cudaError_t e = ensure_dynamic_smem<&gate_logits_kernel>((int)lsm);
-            if (e != cudaSuccess) return e;
-            dim3 grid((D.T + TB - 1) / TB, (D.E + EBL - 1) / EBL);
-            launch_chained(gate_logits_kernel, dim3(grid), dim3(256), lsm, st, D.T, D.E, D.d, x, gate_w, logits_ws, TB, EBL);
+        // Many experts or many tokens: gate logits by the tiled kernel first, then route from those logits.  (Below that a block per
+        // token reads the few gate rows itself: one launch less.)
+        const bool many_tokens = D.T >= 256;      // more blocks than fit at once: throughput counts, not one block's latency
+        if (!logits_in && logits_ws && (D.E > 16 || many_tokens)) {
+            dim3 grid((D.T + GATE_TB - 1) / GATE_TB, (D.E + GATE_EB - 1) / GATE_EB);
+            launch_chained(gate_logits_kernel, dim3(grid), dim3(128), 0, st, D.T, D.E, D.d, x, gate_w, logits_ws);
             logits_in = logits_ws;
             gate_w = nullptr;
         }
-        const size_t smem = row_bytes * (1 + EB) + tail_bytes;
+        // staging area: EB gate rows (or width rows, batch by batch), or the width rows of all selected experts if they fit in half
+        // of what an SM has
+        if (logits_in && forced) EB = 0;
+        int slot_pitch = 0;
+        if (!forced && (size_t)D.k * ((size_t)D.K * row_bytes + 64) + row_bytes + tail_bytes <= 110 * 1024) slot_pitch = D.K * D.d + 32;
+        size_t ws_elems = !EB ? 0 : slot_pitch ? (size_t)D.k * slot_pitch : (size_t)EB * D.d;
+        if (EB && !logits_in && ws_elems < (size_t)EB * D.d) ws_elems = (size_t)EB * D.d;
+        const size_t smem = (EB ? row_bytes : 0) + 2 * ws_elems + tail_bytes;
         cudaError_t e = ensure_dynamic_smem<&route_block_kernel>((int)smem);
         if (e != cudaSuccess) return e;
         // logits and widths both supplied: no dot products, one warp per token does the selection
-        const int threads = (logits_in && forced) ? 32 : 256;
-        launch_chained(route_block_kernel, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB);
+        const int threads = (logits_in && forced) ? 32 : (logits_in && slot_pitch) ? 128 : 256;
+        launch_chained(route_block_kernel, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB,
+                       (int)ws_elems, slot_pitch);
     } else
     launch_chained(route_kernel, dim3((D.T + warps_per_block - 1) / warps_per_block), dim3(warps_per_block * 32), 0, st, 
         D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status);
@@ -417,9 +557,14 @@ cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bf
         launch_chained(group_block_kernel, dim3(blocks), dim3(1024), gsm, st, D.A, n_keys, keys_ws, R.group_off, R.perm, R.inv_perm);
         return cudaGetLastError();
     }
-    launch_chained(count_kernel, dim3((n_keys + 3) / 4), dim3(128), 0, st, D.A, n_keys, keys_ws, hist_ws);
-    launch_chained(scan_kernel, dim3(1), dim3(32), 0, st, n_keys, hist_ws, R.group_off);
-    launch_chained(scatter_kernel, dim3((n_keys + 3) / 4), dim3(128), 0, st, D.A, n_keys, keys_ws, R.group_off, R.perm, R.inv_perm);
+    // runs of at least 512 assignments, as many as the histogram space holds
+    long long n_runs = hist_ints / n_keys < GS_MAX_RUNS ? hist_ints / n_keys : GS_MAX_RUNS;
+    if (n_runs > (D.A + GS_THREADS - 1) / GS_THREADS) n_runs = (D.A + GS_THREADS - 1) / GS_THREADS;
+    const int run = (int)(((D.A + n_runs - 1) / n_runs + GS_THREADS - 1) / GS_THREADS * GS_THREADS);
+    n_runs = (D.A + run - 1) / run;
+    launch_chained(run_rank_kernel, dim3((unsigned)n_runs), dim3(GS_THREADS), (size_t)n_keys * 4, st, D.A, n_keys, run, keys_ws, R.inv_perm, hist_ws);
+    launch_chained(run_place_kernel, dim3((unsigned)n_runs), dim3(GS_THREADS), (size_t)n_keys * 4, st, D.A, n_keys, run, (int)n_runs, keys_ws, hist_ws,
+                   R.group_off, R.perm, R.inv_perm);
     return cudaGetLastError();
 }
 
@@ -494,6 +639,6 @@ extern "C" d2moe_status d2moe_route_static_scratch(const d2moe_config* c, int64_
     RouteBufs R{topk_idx, topk_w, bit_idx, perm, inv_perm, group_off};
     launch_chain_begin();
     cudaError_t e = launch_route(D, (const __nv_bfloat16*)x, (const __nv_bfloat16*)gate_w, logits,
-                                 (const __nv_bfloat16*)bit_w, forced, R, nullptr, keys, hist, device_status, st);
+                                 (const __nv_bfloat16*)bit_w, forced, R, nullptr, keys, hist, D2MOE_STATIC_MAX_KEYS, device_status, st);
     return e == cudaSuccess ? D2MOE_OK : D2MOE_ERR_CUDA;
 }
