@@ -136,6 +136,63 @@ route_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16
     }
 }
 
+// Bit-width choice of every (token, selected expert) pair for many tokens: eight lanes per pair, which read the token's row and
+// the expert's width rows straight from memory (8 bytes per load: lane q carries the chains 4q .. 4q + 3 of the pinned order), four
+// rows at a time.  No shared memory and no barrier, so that all pairs are in flight; bound by the rows' trip from L2.
+// (Staged in shared memory by a block per token, three barriers each: 65 us for 9000 pairs of 3 rows x 2048.)
+__global__ void __launch_bounds__(128)
+width_router_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ bit_w, RouteBufs R,
+                    int32_t* __restrict__ keys) {
+    pdl_enter();
+    const int q = threadIdx.x & 7, a = blockIdx.x * 16 + (threadIdx.x >> 3);
+    const int ac = min(a, D.A - 1), t = ac / D.k, e = R.topk_idx[ac];
+    const uint2* xr = reinterpret_cast<const uint2*>(x + (size_t)t * D.d) + q;
+    const __nv_bfloat16* w0 = bit_w + (size_t)e * D.K * D.d;
+    float best = 0.0f;
+    int kk = 0;
+    for (int c0 = 0; c0 < D.K; c0 += 4) {
+        const uint2* wr[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) wr[r] = reinterpret_cast<const uint2*>(w0 + (size_t)min(c0 + r, D.K - 1) * D.d) + q;
+        const int nr = min(4, D.K - c0);
+        float acc[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[r][j] = 0.0f;
+        const int steps = D.d / 32;
+#pragma unroll 8
+        for (int i = 0; i < steps; ++i) {
+            const uint2 xv = xr[8 * i];
+            const float xf[4] = {__uint_as_float(xv.x << 16), __uint_as_float(xv.x & 0xffff0000u),
+                                 __uint_as_float(xv.y << 16), __uint_as_float(xv.y & 0xffff0000u)};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                if (r < nr) {
+                    const uint2 wv = wr[r][8 * i];
+                    acc[r][0] = fmaf(xf[0], __uint_as_float(wv.x << 16), acc[r][0]);
+                    acc[r][1] = fmaf(xf[1], __uint_as_float(wv.x & 0xffff0000u), acc[r][1]);
+                    acc[r][2] = fmaf(xf[2], __uint_as_float(wv.y << 16), acc[r][2]);
+                    acc[r][3] = fmaf(xf[3], __uint_as_float(wv.y & 0xffff0000u), acc[r][3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {             // butterfly: chain distance 16, 8, 4 is lane distance 4, 2, 1; 2 and 1 are the lane's own
+#pragma unroll
+            for (int off = 4; off; off >>= 1)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[r][j] += __shfl_xor_sync(0xffffffffu, acc[r][j], off);
+            const float v = (acc[r][0] + acc[r][2]) + (acc[r][1] + acc[r][3]);
+            if (c0 + r < D.K && (c0 + r == 0 || v > best)) { best = v; kk = c0 + r; }
+        }
+    }
+    if (q == 0 && a < D.A) {
+        R.bit_idx[a] = (int8_t)kk;
+        keys[a] = e * D.K + kk;
+    }
+}
+
 // Grouping of large loads: a stable counting sort over the grid.  Block b owns a contiguous run of assignments and takes it 32
 // per warp at a time; an assignment's rank among the earlier ones of its key inside the run comes from a match instruction and
 // running counts in shared memory (per warp, then summed over warps: warps own contiguous pieces of each 1024).  Pass 1 leaves
@@ -292,10 +349,10 @@ __device__ __forceinline__ void dots_halfwarp(const uint32_t* x, const uint32_t*
 }
 
 // Gate logits as a tiled product: a block takes 16 tokens x 8 experts, a half-warp forms 4 x 4 of them in registers (same lane
-// layout and order as above), columns stream through shared memory 256 at a time, three stages deep.  Bound: fp32 issue (a
+// layout and order as above), columns stream through shared memory 256 at a time, double buffered (so that nine blocks share an SM).  Bound: fp32 issue (a
 // multiply-add, half a conversion and a quarter of a shared load per product).
 // 1500 tokens x 64 experts x 2048: 62 us before (one dot per warp, two 2-byte shared loads per product).
-constexpr int GATE_TB = 16, GATE_EB = 8, GATE_COLS = 256, GATE_STAGES = 3;
+constexpr int GATE_TB = 16, GATE_EB = 8, GATE_COLS = 256, GATE_STAGES = 2;
 constexpr int GATE_PITCH = GATE_COLS / 2 + 4;           // words per row: four rows on, the other half of the banks
 __global__ void __launch_bounds__(128)
 gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
@@ -319,7 +376,7 @@ gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, con
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    for (int c = 0; c < GATE_STAGES - 1; ++c) stage(c);
+    stage(0);
     float acc[4][4][2];
 #pragma unroll
     for (int t = 0; t < 4; ++t)
@@ -327,9 +384,9 @@ gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, con
         for (int r = 0; r < 4; ++r) acc[t][r][0] = acc[t][r][1] = 0.0f;
     const int xr = (hw & 3) * 4, wr = GATE_TB + (hw >> 2) * 4;
     for (int c = 0; c < n_chunks; ++c) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(GATE_STAGES - 2) : "memory");
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();                          // chunk c is there; the stage refilled next has been read
-        stage(c + GATE_STAGES - 1);
+        stage(c + 1);
         const uint32_t (*b)[GATE_PITCH] = sm[c % GATE_STAGES];
         const int steps = min(GATE_COLS, d - c * GATE_COLS) / 32;
 #pragma unroll 4
@@ -422,7 +479,8 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
     }
     __syncthreads();
 
-    if (!forced && slot_pitch) {       // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
+    const bool later = !forced && slot_pitch < 0;     // the widths are chosen by the next kernel
+    if (!forced && slot_pitch > 0) {   // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
         for (int s = 0; s < D.k; ++s)         // (odd slots half a bank row on: the two half-warps of a warp meet no conflict)
             stage_row(ws + (size_t)s * slot_pitch, bit_w + (size_t)sel_s[s] * D.K * D.d, D.K * D.d);
         stage_wait();
@@ -451,7 +509,7 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
             }
         }
         __syncthreads();
-    } else if (!forced) {       // bit-width router logits of the selected experts: rows (slot s, width c)
+    } else if (!forced && !later) {   // bit-width router logits of the selected experts: rows (slot s, width c)
         const int n_rows = D.k * D.K;
         for (int rb = 0; rb < n_rows; rb += EB) {
             const int n = min(EB, n_rows - rb);
@@ -481,13 +539,14 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
                         if (device_status) atomicOr(device_status, D2MOE_DEV_BAD_INDEX);
                         kk = kk < 0 ? 0 : D.K - 1;
                     }
-                } else {
+                } else if (!later) {
                     float best = u_s[s * D.K];
                     for (int c = 1; c < D.K; ++c)
                         if (u_s[s * D.K + c] > best) { best = u_s[s * D.K + c]; kk = c; }
                 }
                 R.topk_idx[a] = sel[s];
                 R.topk_w[a] = D.renormalize ? w[s] / wsum : w[s];
+                if (later) continue;
                 R.bit_idx[a] = (int8_t)kk;
                 keys[a] = sel[s] * D.K + kk;
             }
@@ -512,8 +571,8 @@ cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bf
     if (EB >= 1 && D.d % 8 == 0) {
         // Many experts or many tokens: gate logits by the tiled kernel first, then route from those logits.  (Below that a block per
         // token reads the few gate rows itself: one launch less.)
-        const bool many_tokens = D.T >= 256;      // more blocks than fit at once: throughput counts, not one block's latency
-        if (!logits_in && logits_ws && (D.E > 16 || many_tokens)) {
+        // 16 experts and fewer: from 1024 tokens on (8 experts x 4096: 22 us either way there).
+        if (!logits_in && logits_ws && (D.E > 16 || D.T >= 1024)) {
             dim3 grid((D.T + GATE_TB - 1) / GATE_TB, (D.E + GATE_EB - 1) / GATE_EB);
             launch_chained(gate_logits_kernel, dim3(grid), dim3(128), 0, st, D.T, D.E, D.d, x, gate_w, logits_ws);
             logits_in = logits_ws;
@@ -522,17 +581,21 @@ cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bf
         // staging area: EB gate rows (or width rows, batch by batch), or the width rows of all selected experts if they fit in half
         // of what an SM has
         if (logits_in && forced) EB = 0;
-        int slot_pitch = 0;
-        if (!forced && (size_t)D.k * ((size_t)D.K * row_bytes + 64) + row_bytes + tail_bytes <= 110 * 1024) slot_pitch = D.K * D.d + 32;
-        size_t ws_elems = !EB ? 0 : slot_pitch ? (size_t)D.k * slot_pitch : (size_t)EB * D.d;
+        // many tokens with their logits at hand: one warp per token selects, the widths are chosen by a kernel of their own
+        const bool later = logits_in && !forced && D.T >= 256;
+        if (later) EB = 0;
+        int slot_pitch = later ? -1 : 0;
+        if (!forced && !later && (size_t)D.k * ((size_t)D.K * row_bytes + 64) + row_bytes + tail_bytes <= 110 * 1024) slot_pitch = D.K * D.d + 32;
+        size_t ws_elems = !EB ? 0 : slot_pitch > 0 ? (size_t)D.k * slot_pitch : (size_t)EB * D.d;
         if (EB && !logits_in && ws_elems < (size_t)EB * D.d) ws_elems = (size_t)EB * D.d;
         const size_t smem = (EB ? row_bytes : 0) + 2 * ws_elems + tail_bytes;
         cudaError_t e = ensure_dynamic_smem<&route_block_kernel>((int)smem);
         if (e != cudaSuccess) return e;
         // logits and widths both supplied: no dot products, one warp per token does the selection
-        const int threads = (logits_in && forced) ? 32 : (logits_in && slot_pitch) ? 128 : 256;
+        const int threads = !EB ? 32 : (logits_in && slot_pitch > 0) ? 128 : 256;
         launch_chained(route_block_kernel, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB,
                        (int)ws_elems, slot_pitch);
+        if (later) launch_chained(width_router_kernel, dim3((D.A + 15) / 16), dim3(128), 0, st, D, x, bit_w, R, keys_ws);
     } else
     launch_chained(route_kernel, dim3((D.T + warps_per_block - 1) / warps_per_block), dim3(warps_per_block * 32), 0, st, 
         D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status);
