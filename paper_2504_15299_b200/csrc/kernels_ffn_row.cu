@@ -1,0 +1,697 @@
+// Grouped dequant-GEMM on the 5th-generation tensor cores (tcgen05 + TMEM) for the expert FFN.
+//
+// One CTA computes, for one (unit, 128-row tile) pair, D[128 weight rows, N tokens] over a range of
+// K-groups.  A "unit" is up to n_cap consecutive columns (tokens) of one expert in the padded,
+// (expert, width)-sorted activation buffer; it holds one piece per routed width, each padded to a
+// multiple of 16 columns.  Weight rows sit on the MMA's M side (TMEM lanes), tokens on N.
+//
+// Per K-group (g input columns) the four dequant warps own one weight row each (thread = row = TMEM
+// lane).  A thread reads its row's packed segments from shared memory and builds the fp16 weights
+// width by width, in registers, using the additivity of the nested code (Section 3.3.1,
+// W_hat_{b_k} = W_hat_{b_1} + sum of the residual terms):
+//     U_0  = (lo - s1/2) + s1 * v_0                       v_j = value of segment j
+//     U_j  = U_{j-1} + M_j * v_j,   M_j = s1 / 2^(bits[j]-bits[0])
+//     W_hat at width bits[j] = U_j + M_j / 2
+// Each step is one AND (isolates a code pair inside the fp16 subnormal range, where a bit pattern
+// v << p is the value v * 2^(p-24)) and one packed half-precision FMA with a pre-scaled multiplier.
+// Every width that has tokens in the unit gets its tile written to TMEM (tcgen05.st) and one
+// tcgen05.mma (A from TMEM, B = the tokens of that width from shared memory) accumulates it into
+// the D columns of those tokens, so each packed byte is read once from HBM however many widths
+// use it (the plane reuse of Section 3.4), and each token is multiplied exactly once.
+// All tiles carry a common power-of-two factor 2^-S (S per matrix, from the largest scale seen at
+// pack time) so that the multipliers stay inside fp16 range; the epilogue multiplies by 2^S.
+//
+// Warp roles (352 threads, 1 CTA per SM, all 512 TMEM columns): warps 0-3 and 4-7 are two dequant
+// warpgroups, each owning one K-half of every tile (thread = weight row = TMEM lane; lanes 2i and 2i + 1
+// hold row i of the tile's two packed blocks, for gate/up the two rows of one hidden unit, which the
+// epilogue pairs with a shuffle) and taking alternate 16-column chunks of the epilogue; warp 8 streams packed blocks (cp.async.bulk), warp 9
+// streams activation tiles (TMA, 128B swizzle, boxes of up to 256 rows), warp 10 issues the MMAs (the
+// whole warp runs the loop, one elected lane issues).  A unit holds up to 320 tokens, so that one
+// dequantization of a weight tile is amortised over enough tensor work to leave the kernel bound by
+// the tensor cores; an MMA covers at most 256 of a piece's columns.  Work items (unit x tile) are taken
+// from a global counter by the weight producer and published to the other warps through a queue in
+// shared memory; the units are ordered by decreasing work.  Every wait is bounded: on expiry
+// the CTA raises D2MOE_DEV_TIMEOUT, stops waiting, drains and exits.
+#include "d2moe_common.cuh"
+#include "kernels_ffn_tc.cuh"
+#include "tc_common.cuh"
+
+#include <type_traits>
+
+namespace {
+
+constexpr int TC_THREADS = 352;        // 8 dequant warps (2 warpgroups) + weight producer + activation producer + MMA issuer
+constexpr int WARP_WPROD = 8, WARP_BPROD = 9, WARP_MMA = 10;
+constexpr int TMEM_COLS = 512;
+constexpr int MAX_SPW = 3;              // operand tiles (64 TMEM columns each, behind the n_cap accumulator columns) per warpgroup
+constexpr int MAX_NSB = 4;              // activation ring depth (upper bound)
+constexpr int MAX_NSW = 6;             // weight ring depth (upper bound; even: a slot always belongs to the same warpgroup)
+constexpr int NSQ = 4;                 // entries of the work queue between the weight producer and the other warps
+
+struct TcParams {
+    MoeDims D;
+    PackLayout L;
+    ExpertPtrs P;
+    int mode;                 // 0: gate/up + SwiGLU -> hbuf;  1: down -> obuf
+    int n_cap, n_row_tiles, n_split, groups_per_split, nsw, nsb, spw;
+    const TcUnit* units;
+    const int* n_units;
+    int* next_item;           // work counter of this launch: starts at the grid size (item i < grid goes to CTA i)
+    __half* hbuf;             // [R, F]
+    float* obuf;              // [n_split][R, d]
+    const float* row_scale;   // [3][R]: per padded row the power-of-two factors of the activation scaling (see tc_gather_kernel)
+    long long R_alloc;
+    int32_t* status;
+    int smem_w_off, smem_bar_off;
+};
+
+// Packed half-precision arithmetic on raw 32-bit registers (a pair of halves each): the running tile lives in plain
+// registers, so nothing is moved between a bit pattern and a half2 value.
+__device__ __forceinline__ uint32_t hfma2_bits(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+__device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// One row's words of a stored segment of SW bits per code: NW words, chunk c at (c*64 + rr)*CS.
+template <int GS, int SW>
+__device__ __forceinline__ void load_row(uint32_t seg, int rr, uint32_t (&w)[GS * SW / 32]) {
+    constexpr int ROW_BYTES = GS * SW / 8;
+    constexpr int CS = ROW_BYTES < 16 ? ROW_BYTES : 16;
+    constexpr int WPL = CS / 4;
+#pragma unroll
+    for (int l = 0; l < ROW_BYTES / CS; ++l) {
+        const uint32_t addr = seg + (uint32_t)((l * D2MOE_TILE_ROWS + rr) * CS);
+        uint32_t* d = w + l * WPL;
+        if constexpr (WPL == 4) {
+            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(addr));
+        } else if constexpr (WPL == 2) {
+            asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(d[0]), "=r"(d[1]) : "r"(addr));
+        } else {
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(d[0]) : "r"(addr));
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Dequantization of one segment of one row into the running tile.
+//   seg     shared-memory address of the segment inside the block
+//   acc     running tile U (GS/2 half2 registers: register i = elements 2i, 2i+1)
+//   m0      multiplier for a code at bit position 0: M_j * 2^(24 - S); position p uses m0 * 2^-p
+//   FIRST   segment 0: the addend is u0 instead of acc
+// ------------------------------------------------------------------------------------------------
+template <int GS, int SW, bool FIRST>
+__device__ __forceinline__ void dequant_segment(uint32_t seg, int rr, uint32_t (&acc)[GS / 2], __half2 m0, __half2 u0) {
+    constexpr int NW = GS * SW / 32;
+    constexpr int PER = 16 / SW;                // registers per word
+    constexpr int NPOS = 8 / SW;                // distinct bit positions per byte lane
+    constexpr uint32_t FIELD = ((1u << SW) - 1u) * 0x00010001u;
+    __half2 mult[NPOS];
+    mult[0] = m0;
+    const __half2 step = __float2half2_rn(1.0f / (float)(1 << SW));     // exact power of two
+#pragma unroll
+    for (int q = 1; q < NPOS; ++q) mult[q] = __hmul2(mult[q - 1], step);
+    uint32_t w[NW];
+    load_row<GS, SW>(seg, rr, w);
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+        const uint32_t lo8 = w[q], hi8 = w[q] >> 8;
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const uint32_t src = (e & 1) ? hi8 : lo8;       // pair e of the word: bytes (0,2) or (1,3), bit SW*(e/2)
+            const int i = q * PER + e;
+            acc[i] = hfma2_bits(src & (FIELD << ((e >> 1) * SW)), as_u32(mult[e >> 1]), FIRST ? as_u32(u0) : acc[i]);
+        }
+    }
+}
+
+// Free residual scales (scale_mode 1): a segment after the first adds SW one-bit steps, each with its own scale, so
+// its codes are folded in bit by bit: U += (2 s_l) bit_l for every step l of the segment (the constant - s_l of
+// W_hat = ... + s_l (2 bit_l - 1) is added when the tile is written).  The bits are a rolled loop: one copy of the code.
+//   sc      shared address of this row's scale of the segment's lowest bit; bit t's lies t planes before
+//   csum    sum of the scales folded in so far, times 2^-S
+template <int GS, int SW>
+__device__ __forceinline__ void dequant_segment_bits(uint32_t seg, uint32_t sc, int rr, uint32_t (&acc)[GS / 2], float two_mS, float& csum) {
+    constexpr int NW = GS * SW / 32;
+    constexpr int PER = 16 / SW;
+    constexpr int NPOS = 8 / SW;
+    uint32_t w[NW];
+    load_row<GS, SW>(seg, rr, w);
+    const __half2 step = __float2half2_rn(1.0f / (float)(1 << SW));
+#pragma unroll 1
+    for (int t = 0; t < SW; ++t) {
+        unsigned short raw;
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(raw) : "r"(sc - (uint32_t)(t * D2MOE_TILE_ROWS * 2)));
+        const float sl = __half2float(__ushort_as_half(raw)) * two_mS;
+        csum += sl;
+        __half2 mult[NPOS];                          // 2 s_l 2^(24 - position)
+        mult[0] = h2dup(sl * __int_as_float((127 + 25 - t) << 23));
+#pragma unroll
+        for (int q = 1; q < NPOS; ++q) mult[q] = __hmul2(mult[q - 1], step);
+        const uint32_t bit = 0x00010001u << t;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const uint32_t lo8 = w[q], hi8 = w[q] >> 8;
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+                const uint32_t src = (e & 1) ? hi8 : lo8;
+                const int i = q * PER + e;
+                acc[i] = hfma2_bits(src & (bit << ((e >> 1) * SW)), as_u32(mult[e >> 1]), acc[i]);
+            }
+        }
+    }
+}
+
+// lane 0's value in every lane: tells the compiler that the value is the same in all lanes, so that what is computed from it
+// stays in uniform registers
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+struct ItemInfo {
+    int unit, tile, split, g0, g1;
+};
+
+__device__ __forceinline__ ItemInfo decode_item(const TcParams& p, int item) {
+    ItemInfo it;
+    const int per_unit = p.n_row_tiles * p.n_split;
+    it.unit = item / per_unit;
+    const int rem = item - it.unit * per_unit;
+    it.tile = rem / p.n_split;
+    it.split = rem - it.tile * p.n_split;
+    it.g0 = it.split * p.groups_per_split;
+    it.g1 = min(p.L.n_groups, it.g0 + p.groups_per_split);
+    return it;
+}
+
+// ------------------------------------------------------------------------------------------------
+// The kernel
+// ------------------------------------------------------------------------------------------------
+// SWS: widths of the stored segments, SWS & 15 that of the first (0: any), SWS >> 4 the sum of the widths that occur later (a
+// code path each); FREE: scale_mode 1.
+template <int GS, int SWS, bool FREE>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMaps maps) {
+    constexpr int HALVES = GS / 64;              // 64-element K slabs of the activation tile
+    constexpr int TILE_COLS = GS / 2;            // TMEM columns of one operand tile
+    extern __shared__ uint8_t smem_raw[];
+    // shared layout (from a 1024-byte boundary, which the 128B-swizzled operand tiles need):
+    // [activation ring: NSB x n_cap*GS*2] [weight ring: nsw x 2 blocks] [barriers]
+    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t smem_base = smem_u32(smem);
+    const uint32_t b_slot_bytes = (uint32_t)p.n_cap * GS * 2;
+    const uint32_t w_slot_bytes = 2u * (uint32_t)p.L.block_bytes;
+    const uint32_t bbuf = smem_base;
+    const uint32_t wbuf = smem_base + p.smem_w_off;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.smem_bar_off);
+    const uint32_t bar0 = smem_u32(bars);
+    auto W_FULL = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+    auto W_EMPTY = [&](int i) { return bar0 + 8u * (uint32_t)(MAX_NSW + i); };
+    auto B_FULL = [&](int i) { return bar0 + 8u * (uint32_t)(2 * MAX_NSW + i); };
+    auto B_EMPTY = [&](int i) { return bar0 + 8u * (uint32_t)(2 * MAX_NSW + MAX_NSB + i); };
+    auto A_FULL = [&](int i) { return bar0 + 8u * (uint32_t)(2 * MAX_NSW + 2 * MAX_NSB + i); };
+    auto A_EMPTY = [&](int i) { return bar0 + 8u * (uint32_t)(2 * MAX_NSW + 2 * MAX_NSB + (2 * MAX_SPW) + i); };
+    const uint32_t D_FULL = bar0 + 8u * (uint32_t)(2 * MAX_NSW + 2 * MAX_NSB + 2 * (2 * MAX_SPW));
+    const uint32_t D_EMPTY = D_FULL + 8u;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_NSW + 2 * MAX_NSB + 2 * (2 * MAX_SPW) + 2);
+    // tail of the 512-byte barrier block, where the waits look for them: device-status pointer (496), abort flag (504)
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bars) + 504);
+    // Work queue (bytes 288..351 and 480..495 of the barrier block): the weight producer takes work items from a global
+    // counter and publishes them to the other warps, so that CTAs that drew cheap items take more of them.
+    // An entry is released by the activation producer, the issuer warp and the eight dequant warps.
+    static_assert(8 * (2 * MAX_NSW + 2 * MAX_NSB + 2 * (2 * MAX_SPW) + 2) + 8 <= 288, "barrier block");
+    auto SQ_FULL = [&](uint32_t i) { return bar0 + 288u + 8u * i; };
+    auto SQ_EMPTY = [&](uint32_t i) { return bar0 + 320u + 8u * i; };
+    volatile int* sq_item = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bars) + 480);
+
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < MAX_NSW; ++i) { mbar_init(W_FULL(i), 1); mbar_init(W_EMPTY(i), 4); }
+        for (int i = 0; i < MAX_NSB; ++i) { mbar_init(B_FULL(i), 1); mbar_init(B_EMPTY(i), 1); }
+        for (int i = 0; i < (2 * MAX_SPW); ++i) { mbar_init(A_FULL(i), 4); mbar_init(A_EMPTY(i), 1); }
+        mbar_init(D_FULL, 1);
+        mbar_init(D_EMPTY, 8);
+        for (int i = 0; i < NSQ; ++i) { mbar_init(SQ_FULL(i), 1); mbar_init(SQ_EMPTY(i), 10); }
+        *abort_flag = 0;
+        *reinterpret_cast<int32_t**>(reinterpret_cast<uint8_t*>(bars) + 496) = p.status;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    // per-width constants of the dequant loop, read from shared memory instead of the kernel parameters
+    // (a dynamically indexed parameter read costs a constant-cache round trip per tile)
+    // per stored segment: {storage width | width index << 8 | last segment of its width << 16, byte offset,
+    // bits of 2^(position - (top - b1)), scale_mode 1: byte offset of the scale of the field's lowest bit}
+    int4* seg_tab = reinterpret_cast<int4*>(reinterpret_cast<uint8_t*>(bars) + 352);
+    if (threadIdx.x < 8) {
+        const int j = threadIdx.x;
+        const int kk = p.L.seg_kk[j];
+        const int last = (j < p.L.n_seg && p.L.last_seg[kk] == j) ? 1 : 0;
+        const int e = p.L.seg_shift[j] - (p.L.top - p.L.b1);
+        const int sc_t0 = p.L.w_sc_off[kk] + ((p.L.top - p.L.b1 - 1 - p.L.seg_shift[j]) - p.L.w_lv0[kk]) * D2MOE_TILE_ROWS * 2;
+        seg_tab[j] = make_int4(p.L.seg_sw[j] | (kk << 8) | (last << 16), p.L.seg_off[j], (127 + e) << 23, sc_t0);
+    }
+    if (warp == WARP_MMA) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = (uint32_t)uniform((int)*tmem_slot);
+    const uint32_t d_tmem = tmem_base;                       // columns [0, n_cap)
+    const uint32_t a_tmem = tmem_base + (uint32_t)p.n_cap;    // 2 spw tiles, 64 columns apart
+
+    // set-up done (barriers, TMEM): from here on the kernel reads what the kernels before it wrote
+    pdl_wait();
+    const int n_units = uniform(*p.n_units);
+    const int total_items = n_units * p.n_row_tiles * p.n_split;
+    const int nsw = p.nsw;
+    // next work item of a consumer: queue entry qi (one arrival per warp, or per thread for a single-thread role)
+    auto pop = [&](uint32_t qi, bool whole_warp) -> int {
+        const uint32_t q = qi & (NSQ - 1);
+        mbar_wait_blk(SQ_FULL(q), (qi / NSQ) & 1u);
+        const int item = sq_item[q];
+        if (whole_warp) __syncwarp();
+        if (!whole_warp || lane == 0) mbar_arrive(SQ_EMPTY(q));
+        return item;
+    };
+
+    if (warp == WARP_WPROD) {
+        // ---------------- weight producer ----------------
+        if (lane == 0) {
+            uint32_t it = 0, wph = 0;
+            int ws = 0;
+            int item = blockIdx.x;
+            for (uint32_t qi = 0;; ++qi) {
+                const uint32_t q = qi & (NSQ - 1);
+                mbar_wait_blk(SQ_EMPTY(q), ((qi / NSQ) & 1u) ^ 1u);
+                if (item >= total_items) item = -1;                    // the end mark
+                sq_item[q] = item;
+                mbar_arrive(SQ_FULL(q));
+                if (item < 0) break;
+                const int next = atomicAdd(p.next_item, 1);            // in flight while this item's blocks are issued
+                const ItemInfo ii = decode_item(p, item);
+                const TcUnit* u = p.units + ii.unit;
+                const int e = u->e, kmax = u->kmax;
+                const uint32_t bytes = (uint32_t)d2moe_prefix_bytes(p.L, kmax);
+                const uint8_t *m0, *m1;
+                int rt0, rt1;
+                if (p.mode == 0) { m0 = p.P.w[3 * e + 0]; m1 = p.P.w[3 * e + 1]; rt0 = rt1 = ii.tile; }
+                else { m0 = m1 = p.P.w[3 * e + 2]; rt0 = 2 * ii.tile; rt1 = 2 * ii.tile + 1; }
+                for (int G = ii.g0; G < ii.g1; ++G, ++it) {
+                    const int s = ws;                                  // ring slot and parity advance by addition
+                    mbar_wait_blk(W_EMPTY(s), wph ^ 1u);
+                    if (*abort_flag) break;                            // nothing more is copied
+                    if (++ws == nsw) { ws = 0; wph ^= 1u; }
+                    mbar_expect_tx(W_FULL(s), 2 * bytes);
+                    const uint32_t dst = wbuf + s * w_slot_bytes;
+                    bulk_g2s(dst, m0 + d2moe_block_offset(p.L, rt0, G), bytes, W_FULL(s));
+                    bulk_g2s(dst + p.L.block_bytes, m1 + d2moe_block_offset(p.L, rt1, G), bytes, W_FULL(s));
+                }
+                item = next;
+            }
+            // drain: every copy issued must have landed before the CTA may exit
+            for (int s = 0; s < nsw && s < (int)it; ++s) {
+                const uint32_t last = it - 1 - (it - 1 - s) % nsw;   // last iteration that used slot s
+                mbar_wait(W_FULL(s), (last / nsw) & 1, abort_flag, p.status, true);
+            }
+        }
+    } else if (warp == WARP_BPROD) {
+        // ---------------- activation producer ----------------
+        if (lane == 0) {
+            uint32_t it = 0, bph = 0;
+            int bs = 0;
+            for (uint32_t qi = 0;; ++qi) {
+                const int item = pop(qi, false);
+                if (item < 0) break;
+                const ItemInfo ii = decode_item(p, item);
+                const TcUnit* u = p.units + ii.unit;
+                const int ncols = u->ncols;                       // multiple of 16, <= n_cap
+                const int row0 = u->row0;                         // read once: the copies below are issued back to back
+                const uint32_t bytes = (uint32_t)ncols * 128u * HALVES;
+                for (int G = ii.g0; G < ii.g1; ++G, ++it) {
+                    const int s = bs;
+                    mbar_wait_blk(B_EMPTY(s), bph ^ 1u);
+                    if (*abort_flag) break;
+                    if (++bs == p.nsb) { bs = 0; bph ^= 1u; }
+                    mbar_expect_tx(B_FULL(s), bytes);
+                    const uint32_t dst = bbuf + s * b_slot_bytes;
+                    // the rows of the unit as boxes of 256, 128, 64, 32, 16 rows (largest first)
+                    int r = 0;
+                    for (int mi = 4; mi >= 0; --mi) {
+                        const int box = 16 << mi;
+                        while (ncols - r >= box) {
+#pragma unroll
+                            for (int h = 0; h < HALVES; ++h)
+                                tma_load_2d(dst + h * (uint32_t)p.n_cap * 128u + (uint32_t)r * 128u, &maps.m[mi],
+                                            G * GS + h * 64, row0 + r, B_FULL(s));
+                            r += box;
+                        }
+                    }
+                }
+            }
+            for (int s = 0; s < p.nsb && s < (int)it; ++s) {
+                const uint32_t last = it - 1 - (it - 1 - s) % p.nsb;
+                mbar_wait(B_FULL(s), (last / p.nsb) & 1, abort_flag, p.status, true);
+            }
+        }
+    } else if (warp == WARP_MMA) {
+        // ---------------- MMA issuer: one thread ----------------
+        // (One thread runs the whole loop: with the warp in the loop and a lane elected around every tile's products, a tile
+        // costs 454 cycles of the issuer next to eight busy warps, this way 299: measured alone, 16-column tiles.)
+        // The issuer is a serial resource (one hand-off per tile), so everything an MMA needs is a register
+        // add away: per item the pieces' instruction descriptors, D columns and row offsets; per stage the low word of the shared-memory
+        // descriptor (its high word is a constant).
+        constexpr uint32_t DESC_HI = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);
+        if (elect_one()) {
+        // sl, ph: next operand slot of either warpgroup and the parity of its wait
+        uint32_t it = 0, sl0 = 0, sl1 = 0, ph0 = 0, ph1 = 0, ic = 0, bph = 0;
+        int bs = 0;
+        const uint32_t spw = (uint32_t)p.spw;
+        const uint32_t slab_step = (uint32_t)p.n_cap * 8u;        // second 64-column slab of a stage, in 16-byte units
+        for (uint32_t qi = 0;; ++qi, ++ic) {
+            const int item = pop(qi, false);
+            if (item < 0) break;
+            const ItemInfo ii = decode_item(p, item);
+            const TcUnit* u = p.units + ii.unit;
+            const int kmax = u->kmax;
+            uint32_t id0[8], dc[8], bo[8];                        // descriptor, D column, B rows / 16 B
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+                const int cnt = kk <= kmax ? u->cnt[kk] : 0;
+                const int col0 = u->col0[kk];
+                id0[kk] = cnt ? instr_desc_f16(cnt) : 0u;
+                dc[kk] = d_tmem + col0;
+                bo[kk] = (uint32_t)col0 * 8u;
+            }
+            mbar_wait_blk(D_EMPTY, (ic & 1) ^ 1);
+            tc_fence_after();
+            for (int G = ii.g0; G < ii.g1; ++G, ++it) {
+                const int s = bs;
+                mbar_wait_blk(B_FULL(s), bph);
+                if (++bs == p.nsb) { bs = 0; bph ^= 1u; }
+                const uint32_t blo = (((bbuf + s * b_slot_bytes) & 0x3FFFFu) >> 4) | (1u << 16);
+                const uint32_t accum = (G != ii.g0) ? 1u : 0u;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    if (id0[kk] == 0u) continue;
+                    const uint32_t slot = (it & 1u) ? spw + sl1 : sl0;
+                    mbar_wait_blk(A_FULL(slot), (it & 1u) ? ph1 : ph0);
+                    tc_fence_after();
+                    {
+                        const uint32_t a_addr = a_tmem + slot * 64;
+                        const uint32_t lo = blo + bo[kk];
+#pragma unroll
+                        for (int j = 0; j < GS / 16; ++j)
+                            tc_mma_ts_lohi(dc[kk], a_addr + j * 8, lo + (j >> 2) * slab_step + (j & 3) * 2, DESC_HI, id0[kk],
+                                           j == 0 ? accum : 1u);
+                        tc_commit(A_EMPTY(slot));
+                    }
+                    if (it & 1u) { if (++sl1 == spw) { sl1 = 0; ph1 ^= 1u; } }
+                    else { if (++sl0 == spw) { sl0 = 0; ph0 ^= 1u; } }
+                }
+                tc_commit(B_EMPTY(s));
+            }
+            tc_commit(D_FULL);
+        }
+        // all MMAs must be complete before TMEM is freed
+        if (ic > 0) mbar_wait(D_FULL, (ic - 1) & 1, abort_flag, p.status, true);
+        }
+        __syncwarp();
+    } else {
+        // ---------------- dequant + epilogue warps: warpgroup wg owns the K-groups of parity wg (counted over the items) ----------------
+        const int wg = warp >> 2;
+        const int r = threadIdx.x & 127;         // row of the tile = TMEM lane
+        // lanes 2i and 2i + 1 hold row i of the tile's first and second packed block (mode 0: the gate and the up row of
+        // one hidden unit, which the epilogue pairs with a shuffle)
+        const int blk = r & 1, rr = r >> 1;
+        const uint32_t lane_addr = ((uint32_t)((warp & 3) * 32)) << 16;
+        uint32_t it = 0, sl = 0, slph = 1, ic = 0;
+        uint32_t wph = 0;                               // weight ring: slot and parity advance by addition
+        int ws = wg;
+        uint32_t acc[GS / 2];                           // the running tile: packed half pairs
+        for (uint32_t qi = 0;; ++qi, ++ic) {
+            const int item = pop(qi, true);
+            if (item < 0) break;
+            const ItemInfo ii = decode_item(p, item);
+            const TcUnit* u = p.units + ii.unit;
+            const int e = u->e, kmax = u->kmax;
+            const uint8_t* mat = p.mode == 0 ? p.P.w[3 * e + blk] : p.P.w[3 * e + 2];
+            const int S = matrix_exponent(mat);
+            const float two_mS = exp2f((float)-S);
+            unsigned present = 0;
+            for (int kk = 0; kk <= kmax; ++kk) present |= (u->cnt[kk] > 0 ? 1u : 0u) << kk;
+            const long long row0 = u->row0;                      // read here: the epilogue must not wait for it
+            const int ncols = u->ncols;
+
+#pragma unroll 1
+            for (int G = ii.g0; G < ii.g1; ++G, ++it) {
+                if ((it & 1u) != (uint32_t)wg) continue;             // the other warpgroup's
+                const int s = ws;
+                mbar_wait_blk(W_FULL(s), wph);
+                ws += 2;
+                if (ws >= nsw) { ws -= nsw; wph ^= 1u; }
+                const uint32_t wb = wbuf + s * w_slot_bytes + blk * p.L.block_bytes;
+                uint32_t meta;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(meta) : "r"(wb + 4u * rr));
+                const __half2 mh = as_h2(meta);
+                const float s1 = __low2float(mh), lo = __high2float(mh);
+                // hands the running tile over as the tile of a width index; addend: what the tile lacks of W_hat 2^-S
+                auto write_tile = [&](float addend) {
+                    const int slot = wg * p.spw + (int)sl;
+                    mbar_wait_blk(A_EMPTY(slot), slph);
+                    tc_fence_after();
+                    const uint32_t dst = a_tmem + slot * 64 + lane_addr;
+                    const uint32_t h = as_u32(h2dup(addend));
+#pragma unroll
+                    for (int c = 0; c < TILE_COLS / 16; ++c) {
+                        uint32_t v[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) v[j] = hadd2_bits(acc[c * 16 + j], h);
+                        tc_st16(dst + c * 16, v);
+                    }
+                    tc_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(A_FULL(slot));
+                    if (++sl == (uint32_t)p.spw) { sl = 0; slph ^= 1u; }
+                };
+                // One copy of every piece of code below (a loop over the stored segments, a path per storage width): the loop
+                // has to stay inside the instruction cache, which holds about a thousand instructions of it.  Straight-line
+                // code for every segment was 1.6 times slower with free scales (three in four stalls: no instruction).
+                float csum = 0.0f;                               // free scales: sum of the scales folded in so far, times 2^-S
+                const int smax = p.L.last_seg[kmax];             // stored segments 0..smax
+                int4 tb = seg_tab[0];
+                // the field's multiplier: s1 2^(position - (top - b1)) 2^-S, and for a code at bit position 0 of its lane
+                // (free scales: a base field's position counts from the base code's lowest bit: the same number)
+                float Ms = s1 * __int_as_float(tb.z) * two_mS;
+                {
+                    const int sw = tb.x & 255;
+                    const uint32_t seg = wb + (uint32_t)tb.y;
+                    const __half2 m0 = h2dup(Ms * 16777216.0f), u0 = h2dup((FREE ? lo : lo - 0.5f * s1) * two_mS);
+                    if constexpr ((SWS & 15) != 0) dequant_segment<GS, SWS & 15, true>(seg, rr, acc, m0, u0);
+                    else {
+                        if (sw == 1) dequant_segment<GS, 1, true>(seg, rr, acc, m0, u0);
+                        else if (sw == 2) dequant_segment<GS, 2, true>(seg, rr, acc, m0, u0);
+                        else if (sw == 4) dequant_segment<GS, 4, true>(seg, rr, acc, m0, u0);
+                        else dequant_segment<GS, 8, true>(seg, rr, acc, m0, u0);
+                    }
+                }
+#pragma unroll 1
+                for (int sj = 0;;) {
+                    // the last field of a width's step sits at that width's unit: half a step completes the tile
+                    if (((tb.x >> 16) & 1) && ((present >> ((tb.x >> 8) & 255)) & 1u)) write_tile(FREE ? -csum : 0.5f * Ms);
+                    if (++sj > smax) break;
+                    tb = seg_tab[sj];
+                    const int sw = tb.x & 255, kk = (tb.x >> 8) & 255;
+                    const uint32_t seg = wb + (uint32_t)tb.y;
+                    Ms = s1 * __int_as_float(tb.z) * two_mS;
+                    if (FREE && kk > 0) {
+                        const uint32_t sc = wb + (uint32_t)tb.w + 2u * rr;       // this row's scale of the field's lowest bit
+                        if ((SWS == 0 || (SWS >> 4 & 1)) && sw == 1) dequant_segment_bits<GS, 1>(seg, sc, rr, acc, two_mS, csum);
+                        if ((SWS == 0 || (SWS >> 4 & 2)) && sw == 2) dequant_segment_bits<GS, 2>(seg, sc, rr, acc, two_mS, csum);
+                        if ((SWS == 0 || (SWS >> 4 & 4)) && sw == 4) dequant_segment_bits<GS, 4>(seg, sc, rr, acc, two_mS, csum);
+                    } else if (!FREE || SWS == 0) {
+                        const __half2 m0 = h2dup(Ms * 16777216.0f);
+                        if ((SWS == 0 || (SWS >> 4 & 1)) && sw == 1) dequant_segment<GS, 1, false>(seg, rr, acc, m0, m0);
+                        if ((SWS == 0 || (SWS >> 4 & 2)) && sw == 2) dequant_segment<GS, 2, false>(seg, rr, acc, m0, m0);
+                        if ((SWS == 0 || (SWS >> 4 & 4)) && sw == 4) dequant_segment<GS, 4, false>(seg, rr, acc, m0, m0);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(W_EMPTY(s));
+            }
+
+            // ---- epilogue: D (128 rows x ncols) -> global; the two warpgroups take alternate 16-column chunks ----
+            // While it runs the tensor pipe is idle, so it is kept short: a warp finishes two chunks at a time (two
+            // independent chains of tensor-memory load, shuffle, SwiGLU and stores), their scale factors are fetched a
+            // pair ahead, and SwiGLU is split between the two threads of a hidden unit (the gate row's thread
+            // finishes the first eight tokens of a chunk, the up row's thread the other eight).  Padding columns
+            // (their activation rows and scale factors are never written) are neither stored nor checked.
+            int pc0[8], pcn[8], prl[8];                          // per piece: first column, columns, real columns
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+                pc0[kk] = u->col0[kk]; pcn[kk] = kk <= kmax ? u->cnt[kk] : 0; prl[kk] = u->real[kk];
+            }
+            auto nreal_of = [&](int c0) -> int {               // real tokens among the 16 columns from c0
+                int nreal = 0;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    const int rel = c0 - pc0[kk];
+                    if (pcn[kk] > 0 && rel >= 0 && rel < pcn[kk]) nreal = min(16, max(0, prl[kk] - rel));
+                }
+                return nreal;
+            };
+            mbar_wait_blk(D_FULL, ic & 1);
+            tc_fence_after();
+            const float two_S = exp2f((float)S);
+            const int keep = blk == 0 ? 0 : 8;
+            // mode 0: xs of the eight tokens this thread finishes, then hq of the same; mode 1: hs of all sixteen
+            auto load_scales = [&](int c0, float4 (&sc)[4]) {
+                const long long grow = row0 + c0;
+                if (p.mode == 0) {
+                    const float4* a = reinterpret_cast<const float4*>(p.row_scale + grow + keep);
+                    const float4* b = reinterpret_cast<const float4*>(p.row_scale + p.R_alloc + grow + keep);
+                    sc[0] = a[0]; sc[1] = a[1]; sc[2] = b[0]; sc[3] = b[1];
+                } else {
+                    const float4* a = reinterpret_cast<const float4*>(p.row_scale + 2 * p.R_alloc + grow);
+                    sc[0] = a[0]; sc[1] = a[1]; sc[2] = a[2]; sc[3] = a[3];
+                }
+            };
+            uint32_t overbits = 0;                               // largest |h| seen, as bits (a NaN above every number)
+            auto finish = [&](int c0, const uint32_t (&v)[16], const float4 (&sc)[4]) {
+                const long long grow = row0 + c0;
+                const int nreal = nreal_of(c0);
+                if (p.mode == 0) {
+                    const float xs[8] = {sc[0].x, sc[0].y, sc[0].z, sc[0].w, sc[1].x, sc[1].y, sc[1].z, sc[1].w};
+                    const float hq[8] = {sc[2].x, sc[2].y, sc[2].z, sc[2].w, sc[3].x, sc[3].y, sc[3].z, sc[3].w};
+                    // exchange with the neighbouring lane (the other row of the hidden unit): the gate thread hands
+                    // over tokens 8..15, the up thread tokens 0..7, already times their own matrix's 2^S
+                    float other_v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        other_v[j] = __shfl_xor_sync(0xffffffffu, __uint_as_float(blk == 0 ? v[8 + j] : v[j]) * two_S, 1);
+                    __half* dst = p.hbuf + (grow + keep) * p.D.F + (long long)ii.tile * 64 + rr;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float mine = __uint_as_float(blk == 0 ? v[j] : v[8 + j]) * two_S * xs[j];
+                        const float other = other_v[j] * xs[j];
+                        const float g = blk == 0 ? mine : other, up = blk == 0 ? other : mine;
+                        float h = __fdividef(g, 1.0f + __expf(-g)) * up * hq[j];
+                        if (keep + j < nreal) {
+                            const uint32_t hb = __float_as_uint(h) & 0x7fffffffu;
+                            overbits = max(overbits, hb);
+                            // beyond fp16 even at the token's own scale (or not a number): stored as zero, call flagged below
+                            if (hb > 0x477fe000u) h = 0.0f;                  // bits of 65504
+                            dst[(long long)j * p.D.F] = __float2half_rn(h);
+                        }
+                    }
+                } else {
+                    const float hs[16] = {sc[0].x, sc[0].y, sc[0].z, sc[0].w, sc[1].x, sc[1].y, sc[1].z, sc[1].w,
+                                          sc[2].x, sc[2].y, sc[2].z, sc[2].w, sc[3].x, sc[3].y, sc[3].z, sc[3].w};
+                    float* dst = p.obuf + (long long)ii.split * p.R_alloc * p.D.d + grow * p.D.d + (long long)ii.tile * 128 + blk * 64 + rr;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (j < nreal) dst[(long long)j * p.D.d] = __uint_as_float(v[j]) * two_S * hs[j];
+                }
+            };
+            float4 sa_next[4], sb_next[4];
+            if (wg * 16 < ncols) load_scales(wg * 16, sa_next);
+            if (wg * 16 + 32 < ncols) load_scales(wg * 16 + 32, sb_next);
+            for (int c0 = wg * 16; c0 < ncols; c0 += 64) {
+                const bool two = c0 + 32 < ncols;
+                uint32_t va[16], vb[16];
+                tc_ld16(d_tmem + lane_addr + c0, va);
+                if (two) tc_ld16(d_tmem + lane_addr + c0 + 32, vb);
+                float4 sa[4], sb[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) { sa[q] = sa_next[q]; sb[q] = sb_next[q]; }
+                if (c0 + 64 < ncols) load_scales(c0 + 64, sa_next);
+                if (c0 + 96 < ncols) load_scales(c0 + 96, sb_next);
+                tc_wait_ld();
+                finish(c0, va, sa);
+                if (two) finish(c0 + 32, vb, sb);
+            }
+            if (p.mode == 0 && overbits > 0x477fe000u && p.status) atomicOr(p.status, D2MOE_DEV_NONFINITE);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(D_EMPTY);
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == WARP_MMA) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_ffn_row(const d2moe_config* c, const MoeDims& D, const PackLayout& Lgu, const PackLayout& Ld,
+                           const ExpertPtrs& P, const TcPlan& pl, const TcBuffers& B, int32_t* device_status, cudaStream_t st, void* const* ev) {
+    auto mark = [&](int i) { if (ev) cudaEventRecord((cudaEvent_t)ev[i], st); };
+    const int sms = device_sm_count();
+    TmaMaps maps_x, maps_h;
+    if (!make_maps(&maps_x, B.xp16, pl.R_alloc, D.d) || !make_maps(&maps_h, B.h16, pl.R_alloc, D.F))
+        return cudaErrorNotSupported;
+
+    for (int mode = 0; mode < 2; ++mode) {
+        TcParams p;
+        p.D = D; p.L = mode == 0 ? Lgu : Ld; p.P = P; p.mode = mode;
+        p.n_cap = pl.n_cap;
+        p.n_row_tiles = mode == 0 ? D.F / 64 : D.d / 128;
+        p.n_split = mode == 0 ? 1 : pl.n_split;
+        p.groups_per_split = mode == 0 ? p.L.n_groups : pl.groups_per_split;
+        p.units = B.units; p.n_units = B.n_units; p.next_item = B.n_units + 1 + mode;
+        p.hbuf = B.h16; p.obuf = B.o32; p.row_scale = B.slot_f; p.R_alloc = pl.R_alloc; p.status = device_status;
+        // accumulator columns + 2 spw operand tiles of 64 <= 512
+        p.spw = pl.n_cap <= 128 ? 3 : 2;
+        p.nsb = pl.n_cap <= 128 ? 4 : (pl.n_cap <= 192 ? 3 : 2);
+        const int b_bytes = p.nsb * pl.n_cap * D.g * 2;
+        const int w_slot = 2 * p.L.block_bytes;
+        const int bar_bytes = 512;
+        const int budget = 224 * 1024;
+        int nsw = (budget - b_bytes - 2 * bar_bytes - 1024) / w_slot;
+        if (nsw > MAX_NSW) nsw = MAX_NSW;
+        nsw &= ~1;
+        if (nsw < 2) return cudaErrorInvalidConfiguration;
+        p.nsw = nsw;
+        p.smem_w_off = b_bytes;
+        p.smem_bar_off = (b_bytes + nsw * w_slot + 511) & ~511;     // 512-byte aligned from the 1024-byte aligned base
+        const int smem_bytes = p.smem_bar_off + bar_bytes + 1024;   // + slack for the 1024-byte alignment
+        mark(mode == 0 ? 1 : 2);
+        // storage widths that occur: that of the first segment and, as a sum, those of the later ones
+        int later = 0;
+        for (int j = 1; j < p.L.n_seg; ++j) later |= p.L.seg_w[j];
+        const int sws = p.L.seg_w[0] | later << 4;
+        auto launch = [&](auto kc) -> cudaError_t {
+            constexpr auto kern = decltype(kc)::value;
+            cudaError_t err = ensure_dynamic_smem<kern>(smem_bytes);
+            if (err != cudaSuccess) return err;
+            launch_chained(kern, dim3(sms), dim3(TC_THREADS), smem_bytes, st, p, mode == 0 ? maps_x : maps_h);
+            return cudaSuccess;
+        };
+#define TC_KERNEL(GS_, SWS_, FREE_) std::integral_constant<decltype(&ffn_row_kernel<GS_, SWS_, FREE_>), &ffn_row_kernel<GS_, SWS_, FREE_>>{}
+#define TC_LAUNCH(GS_, SWS_) (p.L.scale_mode == 1 ? launch(TC_KERNEL(GS_, SWS_, true)) : launch(TC_KERNEL(GS_, SWS_, false)))
+        // a kernel of their own for the lists {2,3,4,8} (base 2, steps of 1, 1, 4) and {2,4,8}: the others take one with a path for
+        // every storage width
+        cudaError_t e;
+        if (D.g == 128 && sws == 0x52) e = TC_LAUNCH(128, 0x52);
+        else if (D.g == 128 && sws == 0x62) e = TC_LAUNCH(128, 0x62);
+        else if (D.g == 128) e = TC_LAUNCH(128, 0);
+        else e = TC_LAUNCH(64, 0);
+#undef TC_LAUNCH
+#undef TC_KERNEL
+        if (e != cudaSuccess) return e;
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}

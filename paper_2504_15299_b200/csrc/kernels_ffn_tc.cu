@@ -970,10 +970,13 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
     // (the 8-bit kernel folds one scale per group into its integer accumulators, which needs the tied residual
     // scales: with free scales every load takes the grouped GEMM)
     pl->decode = (avg <= D2MOE_DECODE_MAX_AVG && c->scale_mode == 0) ? 1 : 0;
+    pl->rows = 0;
     if (pl->decode) {
         pl->n_cap = 32;                      // token slots per unit
     } else {
-        pl->n_cap = 320;
+        // up to about 200 tokens per expert the dequantization bounds either kernel
+        pl->rows = avg <= 200 ? 1 : 0;
+        pl->n_cap = !pl->rows ? 320 : (avg <= 104 ? 128 : 192);
     }
     const long long n_pieces = pl->decode ? (long long)c->n_experts + c->n_shared
                                           : (long long)c->n_experts * c->n_bits + c->n_shared;
@@ -1020,6 +1023,8 @@ cudaError_t launch_ffn_tensor(const d2moe_config* c, const MoeDims& D, const Pac
     launch_chained(tc_prep_kernel, dim3(prep_blocks), dim3(256), prep_smem, st, D, R, pl.n_cap, B.units, B.n_units, B.pad_off, B.row_map, B.src_token,
                    pl.max_units, sms, device_status);
     launch_chained(tc_gather_kernel, dim3(1184), dim3(128), 0, st, D.d, x, B.src_token, B.pad_off, n_keys, B.xp16, B.slot_f, pl.R_alloc, device_status);
+
+    if (pl.rows) return launch_ffn_row(c, D, Lgu, Ld, P, pl, B, device_status, st, ev);
 
     TmaMaps maps_x, maps_h;
     if (!make_maps(&maps_x, B.xp16, pl.R_alloc, D.d) || !make_maps(&maps_h, B.h16, pl.R_alloc, D.F))

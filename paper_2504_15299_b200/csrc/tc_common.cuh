@@ -128,7 +128,8 @@ __device__ __forceinline__ void mbar_wait_blk(uint32_t bar, uint32_t parity) {
         "@q bra WAITB_RETRY;\n\t"
         "st.volatile.shared.u32 [blk+504], 1;\n\t"
         "ld.shared.u64 st, [blk+496];\n\t"
-        "red.global.or.b32 [st], 2;\n"    // D2MOE_DEV_TIMEOUT
+        "setp.ne.u64 q, st, 0;\n\t"
+        "@q red.global.or.b32 [st], 2;\n"    // D2MOE_DEV_TIMEOUT
         "WAITB_DONE:\n\t"
         "}"
         ::"r"(bar), "r"(parity) : "memory");
