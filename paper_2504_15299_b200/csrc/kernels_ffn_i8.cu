@@ -779,13 +779,13 @@ __device__ __forceinline__ int round8(int n) { return (n + 7) & ~7; }
 // multiple of 8 slots; cuts every expert into units of 32 slots; records per unit and segment how many
 // of its slots include the segment, and which blocks of 4 slots hold real tokens.
 // Then orders the units by decreasing work per group, so that the expert kernels, whose CTAs draw work
-// items from a counter, take the cheap ones last; sets both work counters (n_units[1], n_units[2]) to
-// the grid size of those kernels.
+// items from a counter, take the cheap ones last; sets the work counters (n_units[1], n_units[2]) to
+// the grid sizes of those kernels.
 // Shared memory: group_off (E K + 1 ints), per expert its first unit (n_exp + 1 ints), per unit its cost (max_units ints),
 // the padded slot offsets (n_exp + 1 ints).
 __global__ void __launch_bounds__(512)
 i8_prep_kernel(MoeDims D, RouteBufs R, I8Unit* units, int* n_units, int32_t* pad_off, int32_t* row_map,
-               int32_t* src_token, float* kappa, int max_units, int top, int b1, int ffn_grid, int32_t* status,
+               int32_t* src_token, float* kappa, int max_units, int top, int b1, int grid_gu, int grid_d, int32_t* status,
                I8SegMap sm, const int32_t* group_keys) {
     pdl_enter();
     extern __shared__ int32_t s_prep[];
@@ -829,7 +829,7 @@ i8_prep_kernel(MoeDims D, RouteBufs R, I8Unit* units, int* n_units, int32_t* pad
         if (lane == 0) {
             pad_off[n_exp] = carry; s_pad[n_exp] = carry; s_total = carry; unit_off[n_exp] = ucarry;
             n_units[0] = min(ucarry, max_units);
-            n_units[1] = ffn_grid; n_units[2] = ffn_grid;
+            n_units[1] = grid_gu; n_units[2] = grid_d;
         }
     }
     __syncthreads();
@@ -1113,9 +1113,13 @@ cudaError_t launch_ffn_i8(const d2moe_config* c, const MoeDims& D, const PackLay
     float* sigma_h = B.slot_f + 2 * pl.R_alloc;
     int8_t* qx = reinterpret_cast<int8_t*>(B.xp16);
     int8_t* qh = reinterpret_cast<int8_t*>(B.h16);
-    const int q_blocks = (int)(pl.R_alloc < 1184 ? pl.R_alloc : 1184);
+    const int q_blocks = (int)(pl.pad_rows < 1184 ? pl.pad_rows : 1184);
 
-    const int ffn_grid = 2 * device_sm_count();
+    // No more CTAs than work items: an expert has at most one unit that is not full (a small layer's launch is then a few blocks
+    // instead of two per SM).
+    const long long units_most = (D.A < D.E ? D.A : D.E) + D.n_shared + pl.pad_rows / I8_SLOTS;
+    auto grid_of = [&](long long tiles) { const long long n = units_most * tiles; return (int)(n < 2 * device_sm_count() ? n : 2 * device_sm_count()); };
+    const int grid_gu = grid_of(D.F / 64), grid_d = grid_of((long long)(D.d / 128) * pl.n_split);
     size_t prep_smem = (size_t)(D.E * D.K + 1 + n_exp + 1 + pl.max_units + n_exp + 1) * 4;
     if (group_keys) {                       // the grouping's staging area shares the buffer
         const size_t gsm = d2moe_group_is_sortable(D.A, D.E * D.K) ? group_sort_smem_ints(D.A, D.E * D.K, 512 / 32) * 4
@@ -1134,7 +1138,7 @@ cudaError_t launch_ffn_i8(const d2moe_config* c, const MoeDims& D, const PackLay
     sm.n_seg = by_step ? D.K : Lgu.n_seg;
     for (int j = 0; j < 8; ++j) sm.seg_kk[j] = by_step ? j : Lgu.seg_kk[j];
     launch_chained(i8_prep_kernel, dim3(1), dim3(group_keys ? 512 : 256), prep_smem, st, D, R, units, B.n_units, B.pad_off, B.row_map,
-                   B.src_token, kappa, pl.max_units, Lgu.top, Lgu.b1, ffn_grid, device_status, sm, group_keys);
+                   B.src_token, kappa, pl.max_units, Lgu.top, Lgu.b1, grid_gu, grid_d, device_status, sm, group_keys);
     // threads per slot: a quarter of the row's cells, in whole warps
     auto q_threads = [](int n) { const int t = ((n / 4 + I8_QCPT - 1) / I8_QCPT + 31) & ~31; return t < 1024 ? t : 1024; };
     launch_chained(i8_quant_kernel<true>, dim3(q_blocks), dim3(q_threads(D.d)), 0, st, D.d, D.g, pl.R_alloc, x, B.src_token, B.pad_off, n_exp, kappa,
@@ -1183,7 +1187,7 @@ cudaError_t launch_ffn_i8(const d2moe_config* c, const MoeDims& D, const PackLay
             constexpr auto kern = decltype(kc)::value;
             cudaError_t err = ensure_dynamic_smem<kern>(smem_bytes);
             if (err != cudaSuccess) return err;
-            launch_chained(kern, dim3(ffn_grid), dim3(i8_threads(nf)), smem_bytes, st, p, mode == 0 ? maps_x : maps_h);
+            launch_chained(kern, dim3(mode == 0 ? grid_gu : grid_d), dim3(i8_threads(nf)), smem_bytes, st, p, mode == 0 ? maps_x : maps_h);
             return cudaSuccess;
         };
 #define I8_KERNEL(GS_, WP_, NF_) std::integral_constant<decltype(&ffn_i8_kernel<GS_, WP_, NF_>), &ffn_i8_kernel<GS_, WP_, NF_>>{}

@@ -446,6 +446,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
             const float two_mS = exp2f((float)-S);
             unsigned present = 0;
             for (int kk = 0; kk <= kmax; ++kk) present |= (u->cnt[kk] > 0 ? 1u : 0u) << kk;
+            const int smax = p.L.last_seg[kmax];                 // stored segments 0..smax
             const long long row0 = u->row0;                      // read here: the epilogue must not wait for it
             const int ncols = u->ncols;
 
@@ -461,19 +462,26 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
                 asm volatile("ld.shared.u32 %0, [%1];" : "=r"(meta) : "r"(wb + 4u * rr));
                 const __half2 mh = as_h2(meta);
                 const float s1 = __low2float(mh), lo = __high2float(mh);
-                // hands the running tile over as the tile of a width index; addend: what the tile lacks of W_hat 2^-S
-                auto write_tile = [&](float addend) {
+                // Hands the running tile over as the tile of a width index.  The tile lacks a constant of W_hat 2^-S that depends on
+                // the width; the first addend holds the one of the widest tile, which therefore goes out as it is (`plain`), the
+                // others get the difference (`addend`).
+                auto write_tile = [&](float addend, bool plain) {
                     const int slot = wg * p.spw + (int)sl;
                     mbar_wait_blk(A_EMPTY(slot), slph);
                     tc_fence_after();
                     const uint32_t dst = a_tmem + slot * 64 + lane_addr;
-                    const uint32_t h = as_u32(h2dup(addend));
+                    if (plain) {
 #pragma unroll
-                    for (int c = 0; c < TILE_COLS / 16; ++c) {
-                        uint32_t v[16];
+                        for (int c = 0; c < TILE_COLS / 16; ++c) tc_st16(dst + c * 16, *reinterpret_cast<uint32_t (*)[16]>(acc + c * 16));
+                    } else {
+                        const uint32_t h = as_u32(h2dup(addend));
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = hadd2_bits(acc[c * 16 + j], h);
-                        tc_st16(dst + c * 16, v);
+                        for (int c = 0; c < TILE_COLS / 16; ++c) {
+                            uint32_t v[16];
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) v[j] = hadd2_bits(acc[c * 16 + j], h);
+                            tc_st16(dst + c * 16, v);
+                        }
                     }
                     tc_wait_st();
                     tc_fence_before();
@@ -484,8 +492,10 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
                 // One copy of every piece of code below (a loop over the stored segments, a path per storage width): the loop
                 // has to stay inside the instruction cache, which holds about a thousand instructions of it.  Straight-line
                 // code for every segment was 1.6 times slower with free scales (three in four stalls: no instruction).
+                // the widest tile's constant: half a step of its width (free scales: the sum of all steps' scales, which costs more to
+                // form in advance than it saves)
+                const float widest = FREE ? 0.0f : 0.5f * s1 * __int_as_float(seg_tab[smax].z) * two_mS;
                 float csum = 0.0f;                               // free scales: sum of the scales folded in so far, times 2^-S
-                const int smax = p.L.last_seg[kmax];             // stored segments 0..smax
                 int4 tb = seg_tab[0];
                 // the field's multiplier: s1 2^(position - (top - b1)) 2^-S, and for a code at bit position 0 of its lane
                 // (free scales: a base field's position counts from the base code's lowest bit: the same number)
@@ -493,7 +503,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
                 {
                     const int sw = tb.x & 255;
                     const uint32_t seg = wb + (uint32_t)tb.y;
-                    const __half2 m0 = h2dup(Ms * 16777216.0f), u0 = h2dup((FREE ? lo : lo - 0.5f * s1) * two_mS);
+                    const __half2 m0 = h2dup(Ms * 16777216.0f), u0 = h2dup((FREE ? lo : lo - 0.5f * s1) * two_mS + widest);
                     if constexpr ((SWS & 15) != 0) dequant_segment<GS, SWS & 15, true>(seg, rr, acc, m0, u0);
                     else {
                         if (sw == 1) dequant_segment<GS, 1, true>(seg, rr, acc, m0, u0);
@@ -505,7 +515,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
 #pragma unroll 1
                 for (int sj = 0;;) {
                     // the last field of a width's step sits at that width's unit: half a step completes the tile
-                    if (((tb.x >> 16) & 1) && ((present >> ((tb.x >> 8) & 255)) & 1u)) write_tile(FREE ? -csum : 0.5f * Ms);
+                    if (((tb.x >> 16) & 1) && ((present >> ((tb.x >> 8) & 255)) & 1u)) write_tile((FREE ? -csum : 0.5f * Ms) - widest, !FREE && sj == smax);
                     if (++sj > smax) break;
                     tb = seg_tab[sj];
                     const int sw = tb.x & 255, kk = (tb.x >> 8) & 255;

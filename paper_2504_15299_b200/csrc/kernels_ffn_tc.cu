@@ -984,6 +984,7 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
     const long long n_classes = (long long)c->n_experts * c->n_bits + c->n_shared;
     long long pad_rows = pl->decode ? A_tot + 7 * (n_classes < A_tot ? n_classes : A_tot)
                                     : A_tot + 15 * (n_pieces < A_tot ? n_pieces : A_tot);
+    pl->pad_rows = pad_rows;
     pl->R_alloc = ((pad_rows + 255) / 256) * 256 + 256;
     pl->max_units = (int)(c->n_experts + c->n_shared + pl->R_alloc / pl->n_cap + 1);
     // split-K of the down projection: aim for >= 4 work items per resident CTA

@@ -34,6 +34,7 @@ struct TcPlan {
                             //    to the accumulators); 0: grouped fp16 dequant-GEMM (one tile per width, any load)
     int rows;               // 1: grouped GEMM with whole rows per thread (small units), 0: with half rows (large units)
     int n_cap;              // columns per unit
+    long long pad_rows;     // most padded rows any routing of the call can give
     long long R_alloc;      // rows of the padded activation buffers
     int max_units;
     int n_split, groups_per_split;   // split-K of the down projection
