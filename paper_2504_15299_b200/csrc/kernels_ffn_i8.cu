@@ -1113,7 +1113,6 @@ cudaError_t launch_ffn_i8(const d2moe_config* c, const MoeDims& D, const PackLay
     float* sigma_h = B.slot_f + 2 * pl.R_alloc;
     int8_t* qx = reinterpret_cast<int8_t*>(B.xp16);
     int8_t* qh = reinterpret_cast<int8_t*>(B.h16);
-    const int q_blocks = (int)(pl.pad_rows < 1184 ? pl.pad_rows : 1184);
 
     // No more CTAs than work items: an expert has at most one unit that is not full (a small layer's launch is then a few blocks
     // instead of two per SM).
@@ -1139,9 +1138,11 @@ cudaError_t launch_ffn_i8(const d2moe_config* c, const MoeDims& D, const PackLay
     for (int j = 0; j < 8; ++j) sm.seg_kk[j] = by_step ? j : Lgu.seg_kk[j];
     launch_chained(i8_prep_kernel, dim3(1), dim3(group_keys ? 512 : 256), prep_smem, st, D, R, units, B.n_units, B.pad_off, B.row_map,
                    B.src_token, kappa, pl.max_units, Lgu.top, Lgu.b1, grid_gu, grid_d, device_status, sm, group_keys);
-    // threads per slot: a quarter of the row's cells, in whole warps
+    // threads per slot: a quarter of the row's cells, in whole warps; as many blocks as fit at once (a block per slot if they do)
     auto q_threads = [](int n) { const int t = ((n / 4 + I8_QCPT - 1) / I8_QCPT + 31) & ~31; return t < 1024 ? t : 1024; };
-    launch_chained(i8_quant_kernel<true>, dim3(q_blocks), dim3(q_threads(D.d)), 0, st, D.d, D.g, pl.R_alloc, x, B.src_token, B.pad_off, n_exp, kappa,
+    auto q_blocks = [&](int n) { const long long fit = (long long)device_sm_count() * (2048 / q_threads(n) < 32 ? 2048 / q_threads(n) : 32);
+                                 return (unsigned)(pl.pad_rows < fit ? pl.pad_rows : fit); };
+    launch_chained(i8_quant_kernel<true>, dim3(q_blocks(D.d)), dim3(q_threads(D.d)), 0, st, D.d, D.g, pl.R_alloc, x, B.src_token, B.pad_off, n_exp, kappa,
                                                     qx, B.xk_x, sigma_x, device_status);
 
     TmaMaps maps_x, maps_h;
@@ -1173,7 +1174,7 @@ cudaError_t launch_ffn_i8(const d2moe_config* c, const MoeDims& D, const PackLay
         p.smem_bar_off = (p.smem_rec_off + rec_bytes + 511) & ~511;   // 512-byte aligned from the 1024-byte aligned base
         const int smem_bytes = p.smem_bar_off + bar_bytes + 1024;
         if (mode == 1)
-            launch_chained(i8_quant_kernel<false>, dim3(q_blocks), dim3(q_threads(D.F)), 0, st, D.F, D.g, pl.R_alloc, B.h32,
+            launch_chained(i8_quant_kernel<false>, dim3(q_blocks(D.F)), dim3(q_threads(D.F)), 0, st, D.F, D.g, pl.R_alloc, B.h32,
                            B.src_token, B.pad_off, n_exp, kappa, qh, B.xk_h, sigma_h, device_status);
         mark(mode == 0 ? 1 : 2);
         // width lists of at most four segments that have a specialised kernel (nibble j = width of segment j)

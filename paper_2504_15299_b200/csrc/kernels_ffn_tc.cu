@@ -893,38 +893,46 @@ tc_prep_kernel(MoeDims D, RouteBufs R, int n_cap, TcUnit* units, int* n_units, i
 // by row_scale[2] = 2^eh.  A row that holds a NaN or an infinity becomes zeros (scale 0: its outputs
 // are zero) and the call is flagged.  Padding rows are never consumed: a D column depends only on its
 // own token row.
+// A row of up to 4096 elements is read once (16 bytes per load, kept in registers between the maximum and the scaling).
 __global__ void __launch_bounds__(128)
 tc_gather_kernel(int d, const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ src_token,
                  const int32_t* __restrict__ pad_off, int n_keys, __half* __restrict__ xp16,
                  float* __restrict__ row_scale, long long R_alloc, int32_t* status) {
     pdl_enter();
-    __shared__ float s_red[4];
+    constexpr int KEEP = 4;                                         // 16-byte pieces per thread that stay in registers
+    __shared__ uint32_t s_red[2][4];
     const int total_rows = pad_off[n_keys];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n8 = d / 8;
+    int turn = 0;
     for (int row = blockIdx.x; row < total_rows; row += gridDim.x) {
         const int t = src_token[row];
         if (t < 0) continue;
         // eight elements (16 bytes) per thread and step; d is a multiple of 128 on this path
         const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)t * d);
         uint4* dst = reinterpret_cast<uint4*>(xp16 + (size_t)row * d);
-        float amax = 0.0f;
-        int bad = 0;
-        for (int i = threadIdx.x; i < d / 8; i += blockDim.x) {
-            const uint4 v = src[i];
-            const uint32_t* vi = reinterpret_cast<const uint32_t*>(&v);
+        uint4 v[KEEP];
+        // bits of the largest magnitude: they order like unsigned integers, a NaN or an infinity above every finite value
+        uint32_t m = 0;
+        auto largest = [&](const uint4& q) {
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&vi[k]));
-                amax = fmaxf(amax, fmaxf(fabsf(f.x), fabsf(f.y)));
-                bad |= !(fabsf(f.x) < 3.0e38f) | !(fabsf(f.y) < 3.0e38f);
-            }
+            for (int k = 0; k < 4; ++k) m = max(m, max((w[k] << 16) & 0x7fff0000u, w[k] & 0x7fff0000u));
+        };
+#pragma unroll
+        for (int k = 0; k < KEEP; ++k) {
+            const int i = threadIdx.x + k * 128;
+            v[k] = i < n8 ? src[i] : make_uint4(0u, 0u, 0u, 0u);
         }
-        for (int off = 16; off; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-        bad = __syncthreads_or(bad);
-        if (lane == 0) s_red[warp] = amax;
-        __syncthreads();
-        amax = fmaxf(fmaxf(s_red[0], s_red[1]), fmaxf(s_red[2], s_red[3]));
-        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < KEEP; ++k) largest(v[k]);
+        for (int i = threadIdx.x + KEEP * 128; i < n8; i += 128) largest(src[i]);
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) s_red[turn][warp] = m;
+        __syncthreads();                                             // (two buffers in turn: one barrier per row)
+        m = max(max(s_red[turn][0], s_red[turn][1]), max(s_red[turn][2], s_red[turn][3]));
+        turn ^= 1;
+        const float amax = __uint_as_float(m);
+        const bool bad = !(amax < 3.0e38f);
         int e = 4;
         if (amax > 0.0f && !bad) frexpf(amax, &e);                   // amax = m 2^e, 0.5 <= m < 1
         const float mult = bad ? 0.0f : exp2f((float)(4 - e));
@@ -935,19 +943,23 @@ tc_gather_kernel(int d, const __nv_bfloat16* __restrict__ x, const int32_t* __re
             row_scale[2 * R_alloc + row] = exp2f((float)eh);
             if (bad && status) atomicOr(status, D2MOE_DEV_NONFINITE);
         }
-        for (int i = threadIdx.x; i < d / 8; i += blockDim.x) {
-            const uint4 v = src[i];
-            uint4 o;
-            const uint32_t* vi = reinterpret_cast<const uint32_t*>(&v);
-            uint32_t* oi = reinterpret_cast<uint32_t*>(&o);
+        auto scaled = [&](const uint4& q) {
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+            uint32_t o[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&vi[k]));
-                const __half2 h = bad ? __floats2half2_rn(0.0f, 0.0f) : __floats2half2_rn(f.x * mult, f.y * mult);
-                oi[k] = *reinterpret_cast<const uint32_t*>(&h);
+                const __half2 h = bad ? __floats2half2_rn(0.0f, 0.0f)
+                                      : __floats2half2_rn(__uint_as_float(w[k] << 16) * mult, __uint_as_float(w[k] & 0xffff0000u) * mult);
+                o[k] = *reinterpret_cast<const uint32_t*>(&h);
             }
-            dst[i] = o;
+            return make_uint4(o[0], o[1], o[2], o[3]);
+        };
+#pragma unroll
+        for (int k = 0; k < KEEP; ++k) {
+            const int i = threadIdx.x + k * 128;
+            if (i < n8) dst[i] = scaled(v[k]);
         }
+        for (int i = threadIdx.x + KEEP * 128; i < n8; i += 128) dst[i] = scaled(src[i]);
     }
 }
 
@@ -1023,7 +1035,7 @@ cudaError_t launch_ffn_tensor(const d2moe_config* c, const MoeDims& D, const Pac
     const int prep_blocks = supplied || D.A_tot <= 512 ? 1 : (D.A_tot >= 64 * 512 ? 64 : (D.A_tot + 511) / 512);
     launch_chained(tc_prep_kernel, dim3(prep_blocks), dim3(256), prep_smem, st, D, R, pl.n_cap, B.units, B.n_units, B.pad_off, B.row_map, B.src_token,
                    pl.max_units, sms, device_status);
-    launch_chained(tc_gather_kernel, dim3(1184), dim3(128), 0, st, D.d, x, B.src_token, B.pad_off, n_keys, B.xp16, B.slot_f, pl.R_alloc, device_status);
+    launch_chained(tc_gather_kernel, dim3((unsigned)(pl.pad_rows < 16 * sms ? pl.pad_rows : 16 * sms)), dim3(128), 0, st, D.d, x, B.src_token, B.pad_off, n_keys, B.xp16, B.slot_f, pl.R_alloc, device_status);
 
     if (pl.rows) return launch_ffn_row(c, D, Lgu, Ld, P, pl, B, device_status, st, ev);
 
