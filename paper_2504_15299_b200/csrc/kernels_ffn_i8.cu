@@ -350,7 +350,7 @@ ffn_i8_kernel(const __grid_constant__ I8Params p, const __grid_constant__ TmaMap
         // a queue entry is released by the issuer warp, the four unpack warps and the fold warps
         for (int i = 0; i < I8_NSQ; ++i) { mbar_init(SQ_FULL(i), 1); mbar_init(SQ_EMPTY(i), 5 + 4 * NF); }
         *abort_flag = 0;
-        *reinterpret_cast<int32_t**>(reinterpret_cast<uint8_t*>(bars) + 496) = p.status;
+        *reinterpret_cast<int32_t**>(reinterpret_cast<uint8_t*>(bars) + 496) = status_or_sink(p.status);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }

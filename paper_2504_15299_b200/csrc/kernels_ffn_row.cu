@@ -237,7 +237,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
         mbar_init(D_EMPTY, 8);
         for (int i = 0; i < NSQ; ++i) { mbar_init(SQ_FULL(i), 1); mbar_init(SQ_EMPTY(i), 10); }
         *abort_flag = 0;
-        *reinterpret_cast<int32_t**>(reinterpret_cast<uint8_t*>(bars) + 496) = p.status;
+        *reinterpret_cast<int32_t**>(reinterpret_cast<uint8_t*>(bars) + 496) = status_or_sink(p.status);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }

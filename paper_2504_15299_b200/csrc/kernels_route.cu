@@ -424,6 +424,8 @@ gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, con
 // One block (8 warps) per token: the same results as route_kernel, with the token row and batches of
 // EB weight rows staged in shared memory by 16-byte loads (the pinned summation order makes a lane
 // walk a row with stride 32, which is slow straight from global memory); warp w takes row w of a batch.
+// FORCED: the widths are supplied (a kernel of its own: the code for choosing them costs such a call 1 us of instruction fetch).
+template <bool FORCED>
 __global__ void __launch_bounds__(256)
 route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
                    const float* __restrict__ logits_in, const __nv_bfloat16* __restrict__ bit_w,
@@ -479,8 +481,8 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
     }
     __syncthreads();
 
-    const bool later = !forced && slot_pitch < 0;     // the widths are chosen by the next kernel
-    if (!forced && slot_pitch > 0) {   // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
+    const bool later = !FORCED && slot_pitch < 0;     // the widths are chosen by the next kernel
+    if (!FORCED && slot_pitch > 0) {   // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
         for (int s = 0; s < D.k; ++s)         // (odd slots half a bank row on: the two half-warps of a warp meet no conflict)
             stage_row(ws + (size_t)s * slot_pitch, bit_w + (size_t)sel_s[s] * D.K * D.d, D.K * D.d);
         stage_wait();
@@ -509,7 +511,7 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
             }
         }
         __syncthreads();
-    } else if (!forced && !later) {   // bit-width router logits of the selected experts: rows (slot s, width c)
+    } else if (!FORCED && !later) {   // bit-width router logits of the selected experts: rows (slot s, width c)
         const int n_rows = D.k * D.K;
         for (int rb = 0; rb < n_rows; rb += EB) {
             const int n = min(EB, n_rows - rb);
@@ -533,7 +535,7 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
             if (s < D.k) {
                 const int a = t * D.k + s;
                 int kk = 0;
-                if (forced) {
+                if (FORCED) {
                     kk = forced[a];
                     if (kk < 0 || kk >= D.K) {
                         if (device_status) atomicOr(device_status, D2MOE_DEV_BAD_INDEX);
@@ -589,11 +591,11 @@ cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bf
         size_t ws_elems = !EB ? 0 : slot_pitch > 0 ? (size_t)D.k * slot_pitch : (size_t)EB * D.d;
         if (EB && !logits_in && ws_elems < (size_t)EB * D.d) ws_elems = (size_t)EB * D.d;
         const size_t smem = (EB ? row_bytes : 0) + 2 * ws_elems + tail_bytes;
-        cudaError_t e = ensure_dynamic_smem<&route_block_kernel>((int)smem);
+        cudaError_t e = forced ? ensure_dynamic_smem<&route_block_kernel<true>>((int)smem) : ensure_dynamic_smem<&route_block_kernel<false>>((int)smem);
         if (e != cudaSuccess) return e;
         // logits and widths both supplied: no dot products, one warp per token does the selection
         const int threads = !EB ? 32 : (logits_in && slot_pitch > 0) ? 128 : 256;
-        launch_chained(route_block_kernel, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB,
+        launch_chained(forced ? route_block_kernel<true> : route_block_kernel<false>, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB,
                        (int)ws_elems, slot_pitch);
         if (later) launch_chained(width_router_kernel, dim3((D.A + 15) / 16), dim3(128), 0, st, D, x, bit_w, R, keys_ws);
     } else

@@ -103,6 +103,10 @@ __device__ __forceinline__ void mbar_wait_ptx(uint32_t bar, uint32_t parity, uin
         ::"r"(bar), "r"(parity), "r"(abort_addr), "l"(status) : "memory");
 }
 
+// where an expired wait reports when the caller passed no status word
+static __device__ int32_t g_status_sink;
+__device__ __forceinline__ int32_t* status_or_sink(int32_t* status) { return status ? status : &g_status_sink; }
+
 // The same for kernels whose barrier block is 512-byte aligned and keeps the abort flag at byte 504 and
 // the device-status pointer at byte 496 of that block: the slow path finds both from the barrier's own
 // address, so a wait keeps no register alive besides the barrier address and the parity.
@@ -128,8 +132,7 @@ __device__ __forceinline__ void mbar_wait_blk(uint32_t bar, uint32_t parity) {
         "@q bra WAITB_RETRY;\n\t"
         "st.volatile.shared.u32 [blk+504], 1;\n\t"
         "ld.shared.u64 st, [blk+496];\n\t"
-        "setp.ne.u64 q, st, 0;\n\t"
-        "@q red.global.or.b32 [st], 2;\n"    // D2MOE_DEV_TIMEOUT
+        "red.global.or.b32 [st], 2;\n"    // D2MOE_DEV_TIMEOUT
         "WAITB_DONE:\n\t"
         "}"
         ::"r"(bar), "r"(parity) : "memory");
