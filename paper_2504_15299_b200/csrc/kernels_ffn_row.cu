@@ -1,37 +1,39 @@
-// Grouped dequant-GEMM on the 5th-generation tensor cores (tcgen05 + TMEM) for the expert FFN.
+// Grouped dequant-GEMM on the 5th-generation tensor cores for small units: up to 192 tokens of one expert per work item.
 //
-// One CTA computes, for one (unit, 128-row tile) pair, D[128 weight rows, N tokens] over a range of
-// K-groups.  A "unit" is up to n_cap consecutive columns (tokens) of one expert in the padded,
-// (expert, width)-sorted activation buffer; it holds one piece per routed width, each padded to a
-// multiple of 16 columns.  Weight rows sit on the MMA's M side (TMEM lanes), tokens on N.
+// The work items, the nested code and its arithmetic (each width's tile built in registers from the one below, one AND and
+// one packed half-precision FMA per code pair), the item queue and the epilogue are those of ffn_tc_kernel.  With few
+// tokens per unit the products of a tile take a fraction of the time its dequantization takes (16 columns: some 150
+// cycles against 500 per warpgroup), so this kernel is laid out around the dequantization, and ffn_tc_kernel around the
+// products:
+//   * a dequant thread builds a whole row of a K-group (64 registers) and the two warpgroups take alternate groups, where
+//     ffn_tc_kernel gives each warpgroup one K-half of every group.  The per-row work (scale and offset, multipliers, the
+//     field table, one barrier round per tile) is then spent once per row instead of twice, and the warpgroups run a
+//     group apart instead of meeting at every tile;
+//   * each warpgroup has operand tiles of its own (spw: 3 of 64 TMEM columns up to 128 tokens, 2 up to 192: the
+//     accumulators take n_cap columns, the operand tiles the rest of 512), so it runs ahead of the issuer by that
+//     many tiles.  A warpgroup only ever waits on its own slots: a slot shared by both would have been released twice
+//     before the slower one looks, which a one-bit parity cannot tell from not at all;
+//   * the activation ring has 4 stages up to 128 tokens, 3 up to 192, and the weight ring an even number of stages, so that
+//     a stage always belongs to the same warpgroup;
+//   * one copy of every code path: a rolled loop over the stored segments with a branch per storage width, the
+//     one-bit steps of free scales rolled as well.  The loop body must stay inside the instruction cache (about a
+//     thousand instructions); straight-line code per segment took 1.6 times as long with free scales;
+//   * the widest tile goes out of the registers as it is (its half step is part of the first addend);
+//   * one thread issues all products (299 cycles a tile next to eight busy warps, 454 with a lane elected per tile).
 //
-// Per K-group (g input columns) the four dequant warps own one weight row each (thread = row = TMEM
-// lane).  A thread reads its row's packed segments from shared memory and builds the fp16 weights
-// width by width, in registers, using the additivity of the nested code (Section 3.3.1,
-// W_hat_{b_k} = W_hat_{b_1} + sum of the residual terms):
-//     U_0  = (lo - s1/2) + s1 * v_0                       v_j = value of segment j
-//     U_j  = U_{j-1} + M_j * v_j,   M_j = s1 / 2^(bits[j]-bits[0])
-//     W_hat at width bits[j] = U_j + M_j / 2
-// Each step is one AND (isolates a code pair inside the fp16 subnormal range, where a bit pattern
-// v << p is the value v * 2^(p-24)) and one packed half-precision FMA with a pre-scaled multiplier.
-// Every width that has tokens in the unit gets its tile written to TMEM (tcgen05.st) and one
-// tcgen05.mma (A from TMEM, B = the tokens of that width from shared memory) accumulates it into
-// the D columns of those tokens, so each packed byte is read once from HBM however many widths
-// use it (the plane reuse of Section 3.4), and each token is multiplied exactly once.
-// All tiles carry a common power-of-two factor 2^-S (S per matrix, from the largest scale seen at
-// pack time) so that the multipliers stay inside fp16 range; the epilogue multiplies by 2^S.
+// What bounds it: the integer-logic and packed-half pipes that unpack the codes (LOP3, HFMA2 and HADD2 together issue some
+// 2.2 instructions per clock and SM, and the dequant warps keep them there), then the end of an item, where the tensor
+// pipe idles while the accumulators are written (10 to 19 %).  Free residual scales take seven one-bit steps per code
+// where tied ones take three fields.  Measured (layer call, before: ffn_tc_kernel with units of 128 to 320):
+// d 4096, F 14336, 8 experts, top-2, widths {2,3,4,8}, 333 tokens 998 -> 842 us; free scales, 64 tokens 1157 -> 1026 us;
+// 64 experts of F 1408, top-6, 1500 tokens 590 -> 537 us.
 //
-// Warp roles (352 threads, 1 CTA per SM, all 512 TMEM columns): warps 0-3 and 4-7 are two dequant
-// warpgroups, each owning one K-half of every tile (thread = weight row = TMEM lane; lanes 2i and 2i + 1
-// hold row i of the tile's two packed blocks, for gate/up the two rows of one hidden unit, which the
-// epilogue pairs with a shuffle) and taking alternate 16-column chunks of the epilogue; warp 8 streams packed blocks (cp.async.bulk), warp 9
-// streams activation tiles (TMA, 128B swizzle, boxes of up to 256 rows), warp 10 issues the MMAs (the
-// whole warp runs the loop, one elected lane issues).  A unit holds up to 320 tokens, so that one
-// dequantization of a weight tile is amortised over enough tensor work to leave the kernel bound by
-// the tensor cores; an MMA covers at most 256 of a piece's columns.  Work items (unit x tile) are taken
-// from a global counter by the weight producer and published to the other warps through a queue in
-// shared memory; the units are ordered by decreasing work.  Every wait is bounded: on expiry
-// the CTA raises D2MOE_DEV_TIMEOUT, stops waiting, drains and exits.
+// Warp roles (352 threads, 1 CTA per SM, all 512 TMEM columns): warps 0-3 and 4-7 the dequant warpgroups (thread =
+// weight row = TMEM lane; lanes 2i and 2i + 1 hold row i of the tile's two packed blocks, for gate/up the two rows of one
+// hidden unit, which the epilogue pairs with a shuffle), which also take alternate 16-column chunks of the epilogue;
+// warp 8 streams packed blocks (cp.async.bulk), warp 9 activation tiles (TMA, 128B swizzle, boxes of 16 to 256 rows),
+// warp 10 issues the MMAs.  Every wait is bounded: on expiry the CTA raises D2MOE_DEV_TIMEOUT, stops waiting, drains
+// and exits.
 #include "d2moe_common.cuh"
 #include "kernels_ffn_tc.cuh"
 #include "tc_common.cuh"
@@ -64,19 +66,6 @@ struct TcParams {
     int32_t* status;
     int smem_w_off, smem_bar_off;
 };
-
-// Packed half-precision arithmetic on raw 32-bit registers (a pair of halves each): the running tile lives in plain
-// registers, so nothing is moved between a bit pattern and a half2 value.
-__device__ __forceinline__ uint32_t hfma2_bits(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t d;
-    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
-__device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
 
 // One row's words of a stored segment of SW bits per code: NW words, chunk c at (c*64 + rr)*CS.
 template <int GS, int SW>
@@ -166,10 +155,6 @@ __device__ __forceinline__ void dequant_segment_bits(uint32_t seg, uint32_t sc, 
         }
     }
 }
-
-// lane 0's value in every lane: tells the compiler that the value is the same in all lanes, so that what is computed from it
-// stays in uniform registers
-__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 struct ItemInfo {
     int unit, tile, split, g0, g1;
@@ -663,7 +648,7 @@ cudaError_t launch_ffn_row(const d2moe_config* c, const MoeDims& D, const PackLa
         p.hbuf = B.h16; p.obuf = B.o32; p.row_scale = B.slot_f; p.R_alloc = pl.R_alloc; p.status = device_status;
         // accumulator columns + 2 spw operand tiles of 64 <= 512
         p.spw = pl.n_cap <= 128 ? 3 : 2;
-        p.nsb = pl.n_cap <= 128 ? 4 : (pl.n_cap <= 192 ? 3 : 2);
+        p.nsb = pl.n_cap <= 128 ? 4 : 3;
         const int b_bytes = p.nsb * pl.n_cap * D.g * 2;
         const int w_slot = 2 * p.L.block_bytes;
         const int bar_bytes = 512;

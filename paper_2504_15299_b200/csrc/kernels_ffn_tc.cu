@@ -1,11 +1,13 @@
-// Grouped dequant-GEMM on the 5th-generation tensor cores (tcgen05 + TMEM) for the expert FFN.
+// Grouped dequant-GEMM on the 5th-generation tensor cores (tcgen05 + TMEM) for the expert FFN: the unit build and the
+// gather of every load beyond the 8-bit decode kernel's, and the kernel of large units (more than about 160 tokens per
+// expert on average; smaller ones go to ffn_row_kernel, see tc_plan).
 //
 // One CTA computes, for one (unit, 128-row tile) pair, D[128 weight rows, N tokens] over a range of
 // K-groups.  A "unit" is up to n_cap consecutive columns (tokens) of one expert in the padded,
 // (expert, width)-sorted activation buffer; it holds one piece per routed width, each padded to a
 // multiple of 16 columns.  Weight rows sit on the MMA's M side (TMEM lanes), tokens on N.
 //
-// Per K-group (g input columns) the four dequant warps own one weight row each (thread = row = TMEM
+// Per K-group (g input columns) a dequant thread owns (half of) one weight row (thread = row = TMEM
 // lane).  A thread reads its row's packed segments from shared memory and builds the fp16 weights
 // width by width, in registers, using the additivity of the nested code (Section 3.3.1,
 // W_hat_{b_k} = W_hat_{b_1} + sum of the residual terms):
@@ -65,19 +67,6 @@ struct TcParams {
     int32_t* status;
     int smem_w_off, smem_bar_off;
 };
-
-// Packed half-precision arithmetic on raw 32-bit registers (a pair of halves each): the running tile lives in plain
-// registers, so nothing is moved between a bit pattern and a half2 value.
-__device__ __forceinline__ uint32_t hfma2_bits(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t d;
-    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
-__device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
 
 // ------------------------------------------------------------------------------------------------
 // Dequantization of one K-half of one segment of one row into the running tile.
@@ -986,9 +975,16 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
     if (pl->decode) {
         pl->n_cap = 32;                      // token slots per unit
     } else {
-        // up to about 200 tokens per expert the dequantization bounds either kernel
-        pl->rows = avg <= 200 ? 1 : 0;
-        pl->n_cap = !pl->rows ? 320 : (avg <= 104 ? 128 : 192);
+        // Small units are bound by the dequantization: ffn_row_kernel does less of it per tile, but its operand tiles leave
+        // room for 128 columns (three tiles a warpgroup) or 192 (two), where ffn_tc_kernel takes 320.  An expert that
+        // outgrows its unit is dequantized once more, so the lines lie where the average load leaves two to three standard
+        // deviations of room: 3/4 of 128 and 5/6 of 192.  Layer call on the Mixtral shape with units of 128 / 192 /
+        // 320: 90 tokens per expert 847 / 905 / 1000 us, 100: 957 / 914 / 1008, 150: 1213 / 967 / 1040, 160: - / 1037 / 1046,
+        // 170: - / 1137 / 1052; 64 experts of F 1408: 150 - / 532 / 568, 169 - / 604 / 607, 178 - / 651 / 630.  With free
+        // scales two operand tiles a warpgroup are too few (75: 1080 / 1278 / 1223, 100: 1283 / 1296 / 1240, 150: 1604 /
+        // 1340 / 1267): units of 128 or of 320.
+        pl->n_cap = avg <= 96 ? 128 : (avg <= 160 && c->scale_mode == 0 ? 192 : 320);
+        pl->rows = pl->n_cap <= 192 ? 1 : 0;
     }
     const long long n_pieces = pl->decode ? (long long)c->n_experts + c->n_shared
                                           : (long long)c->n_experts * c->n_bits + c->n_shared;
@@ -998,7 +994,8 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
                                     : A_tot + 15 * (n_pieces < A_tot ? n_pieces : A_tot);
     pl->pad_rows = pad_rows;
     pl->R_alloc = ((pad_rows + 255) / 256) * 256 + 256;
-    pl->max_units = (int)(c->n_experts + c->n_shared + pl->R_alloc / pl->n_cap + 1);
+    // (grouped GEMM: as if every unit held 128 columns, so that the workspace never shrinks when T grows)
+    pl->max_units = (int)(c->n_experts + c->n_shared + pl->R_alloc / (pl->decode ? pl->n_cap : 128) + 1);
     // split-K of the down projection: aim for >= 4 work items per resident CTA
     long long units_est = (c->n_experts < A ? c->n_experts : A) + (long long)c->n_shared * ((T + pl->n_cap - 1) / pl->n_cap);
     // prefill-sized loads: an expert spans several units (every partial output plane is written by the down

@@ -202,6 +202,24 @@ __device__ __forceinline__ __half2 h2dup(float v) { return __float2half2_rn(v); 
 __device__ __forceinline__ __half2 as_h2(uint32_t u) { return *reinterpret_cast<__half2*>(&u); }
 __device__ __forceinline__ uint32_t as_u32(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
 
+// Packed half-precision arithmetic on raw 32-bit registers (a pair of halves each): the running tile lives in plain
+// registers, so nothing is moved between a bit pattern and a half2 value.
+__device__ __forceinline__ uint32_t hfma2_bits(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+__device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// lane 0's value in every lane: tells the compiler that the value is the same in all lanes, so that what is computed from it
+// stays in uniform registers
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+
 // Compile-time description of a width list of at most four widths: nibble j of WPACK is the width of step j
 // (bits[j] - bits[j-1]; sw: the width of the field it is stored in when that is a single field).  WPACK == 0
 // selects the run-time path.
