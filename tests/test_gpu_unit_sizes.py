@@ -1,0 +1,69 @@
+"""Sizes at which a call changes kernel: the unit width of the grouped GEMM (average tokens per expert 40 | 41, 96 | 97,
+160 | 161) and the routing kernels of large batches, each on both sides of its line."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2504_15299_b200 import synth
+from tests.helpers import np_f32
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2504_15299_b200 import binding, build
+    build.build_library()
+    binding.lib()
+    return binding
+
+
+@pytest.mark.parametrize("scale_mode", [0, 1])
+@pytest.mark.parametrize("g,bits", [(128, (2, 3, 4, 8)), (128, (2, 4, 8)), (64, (3, 5))])
+def test_grouped_gemm_on_both_sides_of_every_unit_width(B, g, bits, scale_mode):
+    # Six experts, top-3: T = 2 * average.  One expert takes every token (more than a unit), the last few tokens;
+    # a rare width gives pieces of a token or two.  Bound: 1e-2 of the row's largest output against the CUDA-core path
+    # on the same packed weights, the bound of the batch-size sweep (two roundings to fp16 and one to bf16, or the
+    # two-term 8-bit operands, all below 2^-8 of a row's maximum).
+    d, F, E, k = 256, 384, 6, 3
+    cfg_tc, cfg_cc = (B.Config(d, F, E, k, g, bits, scale_mode=scale_mode, kernel_path=p) for p in (0, 1))
+    blobs = [B.pack_mwq(cfg_tc, synth.normal(31, 3 * e + m, (F, d) if m < 2 else (d, F), 0.02, "cuda"))
+             for e in range(E) for m in range(3)]
+    rare = [0.02] + [0.98 / (len(bits) - 1)] * (len(bits) - 1)
+    for T in (80, 82, 192, 194, 320, 322):
+        x = synth.bf16_exact(synth.normal(31, 1000 + T, (T, d), 1.0, "cuda"))
+        logits = synth.normal(31, 2000 + T, (T, E), 1.0, "cuda") + torch.tensor([50.0, 0, 0, 0, 0, -2.5], device="cuda")
+        fb = synth.categorical(31, 3000 + T, (T, k), rare, "cuda")
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        y1, y1b = (B.moe_forward(cfg_tc, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st) for _ in range(2))
+        y2 = B.moe_forward(cfg_cc, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st).float()
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        assert torch.equal(y1.view(torch.int16), y1b.view(torch.int16)), ("rerun differs", T)
+        err = float(((y1.float() - y2).abs().amax(dim=1) / y2.abs().amax(dim=1)).max())
+        assert err <= 1e-2, (T, err)
+
+
+@pytest.mark.parametrize("T,E,k,d", [(255, 20, 3, 192), (257, 20, 3, 192),      # tiled gate logits (E > 16), width router (T >= 256)
+                                     (1023, 5, 2, 320), (1029, 5, 2, 320),      # tiled gate logits from 1024 tokens
+                                     (6149, 8, 2, 64), (1100, 64, 6, 64)])      # grouping over the grid: many assignments, many keys
+@pytest.mark.parametrize("forced", [False, True])
+def test_routing_of_large_batches_matches_the_oracle(B, T, E, k, d, forced):
+    from oracle import routing
+    bits = (2, 3, 4, 8)
+    cfg = B.Config(d, 128, E, k, 64, bits)
+    x = synth.bf16_exact(synth.normal(32, T, (T, d), 1.0, "cuda"))
+    gw = synth.bf16_exact(synth.normal(32, 1, (E, d), 0.1, "cuda"))
+    bw = None if forced else synth.bf16_exact(synth.normal(32, 2, (E, len(bits), d), 0.1, "cuda"))
+    fb = synth.categorical(32, 3, (T, k), [0.1, 0.2, 0.4, 0.3], "cuda") if forced else None
+    r = B.route(cfg, x, gate_w=gw, bit_w=bw, forced_bit_idx=fb)
+    torch.cuda.synchronize()
+    ref = routing.route(np_f32(x), E=E, K=len(bits), top_k=k, renormalize=bool(cfg.renormalize), gate_w=np_f32(gw),
+                        bit_w=None if forced else np_f32(bw), forced_bit_idx=fb.cpu().numpy() if forced else None)
+    assert int(r.device_status.item()) == 0
+    assert np.array_equal(r.topk_idx.cpu().numpy(), ref.topk_idx)
+    assert np.array_equal(r.bit_idx.cpu().numpy(), ref.bit_idx)
+    assert np.array_equal(r.perm.cpu().numpy(), ref.grouping.perm)
+    assert np.array_equal(r.inv_perm.cpu().numpy(), ref.grouping.inv_perm)
+    assert np.array_equal(r.group_off.cpu().numpy(), ref.grouping.group_off)
+    assert np.allclose(r.topk_w.cpu().numpy(), ref.topk_w, rtol=1e-5, atol=1e-7)
