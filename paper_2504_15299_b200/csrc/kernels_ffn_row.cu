@@ -676,9 +676,13 @@ cudaError_t launch_ffn_row(const d2moe_config* c, const MoeDims& D, const PackLa
 #define TC_KERNEL(GS_, SWS_, FREE_) std::integral_constant<decltype(&ffn_row_kernel<GS_, SWS_, FREE_>), &ffn_row_kernel<GS_, SWS_, FREE_>>{}
 #define TC_LAUNCH(GS_, SWS_) (p.L.scale_mode == 1 ? launch(TC_KERNEL(GS_, SWS_, true)) : launch(TC_KERNEL(GS_, SWS_, false)))
         // a kernel of their own for the lists {2,3,4,8} (base 2, steps of 1, 1, 4) and {2,4,8}: the others take one with a path for
-        // every storage width
+        // every storage width.  `sws` does not say where the base ends: the list {3,8} has the same one as {2,3,4,8}, but its base
+        // is the first two fields.  With tied scales that is all one; with free scales the two kernels fold every field
+        // after the first bit by bit, so a base of more than one field goes to the general kernel.
+        const bool one_field_base = p.L.scale_mode == 0 || p.L.last_seg[0] == 0;
         cudaError_t e;
-        if (D.g == 128 && sws == 0x52) e = TC_LAUNCH(128, 0x52);
+        if (!one_field_base && D.g == 128) e = TC_LAUNCH(128, 0);
+        else if (D.g == 128 && sws == 0x52) e = TC_LAUNCH(128, 0x52);
         else if (D.g == 128 && sws == 0x62) e = TC_LAUNCH(128, 0x62);
         else if (D.g == 128) e = TC_LAUNCH(128, 0);
         else e = TC_LAUNCH(64, 0);

@@ -44,6 +44,33 @@ def test_grouped_gemm_on_both_sides_of_every_unit_width(B, g, bits, scale_mode):
         assert err <= 1e-2, (T, err)
 
 
+@pytest.mark.parametrize("scale_mode", [0, 1])
+@pytest.mark.parametrize("bits", [(3, 8), (3, 4, 8), (3, 7), (3, 7, 8), (3, 5), (5, 6, 7, 8)])
+def test_base_width_stored_as_two_fields(B, bits, scale_mode):
+    # A base of 3 bits is stored as fields of 2 + 1 bits, one of 5 bits as 4 + 1: the later field still belongs to the base.
+    # Against the oracle (1e-2 of the row's largest output, the suite's bound for bf16 outputs) in the decode kernel, the
+    # small-unit and the large-unit kernel, and in the CUDA-core path.
+    from oracle import moe, mwq, routing
+    d, F, E, k, g = 256, 384, 4, 2, 128
+    cfgs = [B.Config(d, F, E, k, g, bits, scale_mode=scale_mode, kernel_path=p) for p in (0, 1)]
+    Ws = [synth.normal(33, 3 * e + m, (F, d) if m < 2 else (d, F), 0.02, "cuda") for e in range(E) for m in range(3)]
+    blobs = [B.pack_mwq(cfgs[0], W) for W in Ws]
+    triples = [tuple(mwq.quantize(np_f32(Ws[3 * e + m]), bits, g, scale_mode) for m in range(3)) for e in range(E)]
+    for T in (10, 120, 400):
+        x = synth.bf16_exact(synth.normal(33, 1000 + T, (T, d), 1.0, "cuda"))
+        logits = synth.normal(33, 2000 + T, (T, E), 1.0, "cuda")
+        fb = synth.categorical(33, 3000 + T, (T, k), [1.0 / len(bits)] * len(bits), "cuda")
+        rt = routing.route(np_f32(x), E=E, K=len(bits), top_k=k, renormalize=True, logits=np_f32(logits),
+                           forced_bit_idx=fb.cpu().numpy())
+        ref = moe.moe_layer(np_f32(x), rt, lambda e: triples[e], bits, E)
+        for cfg in cfgs:
+            st = torch.zeros(1, dtype=torch.int32, device="cuda")
+            y = np_f32(B.moe_forward(cfg, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st))
+            assert int(st.item()) == 0
+            err = max(float(np.abs(y[t] - ref[t]).max() / np.abs(ref[t]).max()) for t in range(T))
+            assert err <= 1e-2, (T, cfg.kernel_path, err)
+
+
 @pytest.mark.parametrize("T,E,k,d", [(255, 20, 3, 192), (257, 20, 3, 192),      # tiled gate logits (E > 16), width router (T >= 256)
                                      (1023, 5, 2, 320), (1029, 5, 2, 320),      # tiled gate logits from 1024 tokens
                                      (6149, 8, 2, 64), (1100, 64, 6, 64)])      # grouping over the grid: many assignments, many keys
