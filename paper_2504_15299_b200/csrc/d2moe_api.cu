@@ -206,6 +206,24 @@ extern "C" size_t d2moe_workspace_bytes(const d2moe_config* c, int64_t max_token
         d2moe_carve_workspace(c, t_dec, &ws);
         if (ws.total > total) total = ws.total;
     }
+    // free scales: the grouped GEMM takes every batch, also the smallest, and the split of its down projection over K (hence
+    // the space for the partial outputs) falls in steps as the batch grows: cover the last batch of every step.
+    // (Larger batches than t_dec carry the split of t_dec + 1; with tied scales the decode kernel carries that of one token.)
+    if (c->scale_mode == 1 && use_tensor_path(c)) {
+        auto split = [&](long long t) { TcPlan pl; tc_plan(c, t, &pl); return pl.n_split; };
+        const long long most = t_dec < T ? t_dec : T;
+        for (long long t = 1; t <= most; ++t) {
+            const int s = split(t);
+            long long up = most;
+            while (t < up) {
+                const long long mid = (t + up + 1) / 2;
+                if (split(mid) == s) t = mid;
+                else up = mid - 1;
+            }
+            d2moe_carve_workspace(c, t, &ws);
+            if (ws.total > total) total = ws.total;
+        }
+    }
     return total;
 }
 

@@ -994,7 +994,7 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
                                     : A_tot + 15 * (n_pieces < A_tot ? n_pieces : A_tot);
     pl->pad_rows = pad_rows;
     pl->R_alloc = ((pad_rows + 255) / 256) * 256 + 256;
-    // (grouped GEMM: as if every unit held 128 columns, so that the workspace never shrinks when T grows)
+    // (grouped GEMM: as if every unit held 128 columns, so that the unit list never shrinks when T grows)
     pl->max_units = (int)(c->n_experts + c->n_shared + pl->R_alloc / (pl->decode ? pl->n_cap : 128) + 1);
     // split-K of the down projection: aim for >= 4 work items per resident CTA
     long long units_est = (c->n_experts < A ? c->n_experts : A) + (long long)c->n_shared * ((T + pl->n_cap - 1) / pl->n_cap);

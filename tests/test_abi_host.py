@@ -138,3 +138,16 @@ def test_static_scratch_routing_refuses_what_its_array_cannot_hold(lib):
     too_many_tokens = binding.STATIC_MAX_ASSIGNMENTS // c.top_k + 1
     assert lib.d2moe_route_static_scratch(ctypes.byref(c), too_many_tokens, *args) == 5
     assert binding.STATIC_MAX_KEYS == 256 * 8
+
+
+@pytest.mark.parametrize("scale_mode", [0, 1])
+@pytest.mark.parametrize("d,F,E,k,n_shared,g", [(4096, 14336, 8, 2, 0, 128), (2048, 1408, 64, 6, 2, 128), (4096, 1024, 32, 2, 0, 128),
+                                                (2048, 1536, 4, 1, 2, 64), (512, 1408, 1, 1, 0, 64), (128, 14336, 256, 8, 4, 128)])
+def test_workspace_for_max_tokens_serves_every_smaller_batch(lib, d, F, E, k, n_shared, g, scale_mode):
+    # a call of t tokens needs at most workspace_bytes(t), so sizes that never fall with t are enough
+    cfg = binding.Config(d, F, E, k, g, (2, 3, 4, 8), n_shared=n_shared, scale_mode=scale_mode)
+    tokens = sorted(set(range(1, 700)) | {40 * E // k + i for i in (-1, 0, 1, 2)} | {1000, 5000, 20000})
+    tokens = [t for t in tokens if t >= 1]
+    sizes = [binding.workspace_bytes(cfg, t) for t in tokens]
+    falls = [(tokens[i + 1], sizes[i], sizes[i + 1]) for i in range(len(sizes) - 1) if sizes[i] > sizes[i + 1]]
+    assert not falls, falls[:3]
