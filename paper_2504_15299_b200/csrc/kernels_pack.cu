@@ -290,7 +290,8 @@ pack_tied_kernel(PackLayout L, const float* __restrict__ W, uint8_t* __restrict_
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int r = ((p0 + b0 + h) * 8 + warp) * RPW + sub;
-                const bool live = (long long)rt * D2MOE_TILE_ROWS + r < L.rows;
+                // (a one-bit base whose range exceeds fp16: the scale is infinite, its reciprocal 0, no residual a number, every bit 0)
+                const bool live = (long long)rt * D2MOE_TILE_ROWS + r < L.rows && inv[h] > 0.0f;
                 const unsigned long long k2 = pair(inv[h] * two_nl, inv[h] * two_nl);
 #pragma unroll
                 for (int v = 0; v < V; ++v) {
@@ -382,9 +383,12 @@ __device__ __forceinline__ void free_codes(const float (&w)[R][E], float levels,
     }
     const uint32_t flip = (1u << n_lv) - 1u;
 #pragma unroll
-    for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r) {
+        // an infinite base scale (a one-bit base whose range exceeds fp16) leaves no residual that is a number: every bit 0
+        const bool finite = !__hisinf(__low2half(meta[r]));
 #pragma unroll
-        for (int e = 0; e < E; ++e) code[r][e] ^= flip;
+        for (int e = 0; e < E; ++e) code[r][e] = finite ? code[r][e] ^ flip : 0u;
+    }
 }
 
 // Free scales, no error compensation.  One block per packed block; a warp takes four rows at a time.  col_energy

@@ -52,3 +52,25 @@ def test_pack_unaligned_matrix_and_large_offsets(B, g):
     codes, s1, lo = B.unpack_codes(cfg, blob, rows, cols, 8)
     assert np.array_equal(codes.cpu().numpy(), q.code)
     assert np.array_equal(np_f32(s1), q.s1) and np.array_equal(np_f32(lo), q.lo)
+
+
+@pytest.mark.parametrize("scale_mode", [0, 1])
+@pytest.mark.parametrize("g", [32, 64, 128, 256])
+@pytest.mark.parametrize("bits", [(1, 8), (1, 2, 3), (1,)])
+def test_pack_range_beyond_the_scale_format(B, bits, g, scale_mode):
+    # a base of one bit takes the whole range of a group as its scale, which fp16 does not hold from 65520 on: no residual is
+    # a number then and every bit is 0
+    from oracle import mwq
+    rows, cols = 67, 512
+    cfg = B.Config(cols, cols, 2, 1, g, bits, scale_mode=scale_mode)
+    W = synth.normal(19, 5, (rows, cols), 0.02, "cuda")
+    W[3, 0], W[3, 1], W[66, 300], W[66, 301], W[8, 7] = 65000.0, -65000.0, 40000.0, -30000.0, 65503.0
+    blob = B.pack_mwq(cfg, W)
+    with np.errstate(all="ignore"):
+        q = mwq.quantize(np_f32(W), bits, g, scale_mode)
+    assert np.isinf(q.s1).sum() == 2
+    codes, s1, lo = B.unpack_codes(cfg, blob, rows, cols, bits[-1])
+    assert np.array_equal(codes.cpu().numpy(), q.code)
+    assert np.array_equal(np_f32(s1), q.s1) and np.array_equal(np_f32(lo), q.lo)
+    if scale_mode and bits[-1] > bits[0]:
+        assert np.array_equal(np_f32(B.unpack_scales(cfg, blob, rows, cols)), q.s_extra, equal_nan=True)
