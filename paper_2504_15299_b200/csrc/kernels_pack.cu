@@ -325,13 +325,14 @@ __device__ __forceinline__ void free_codes(const float (&w)[R][E], float levels,
                                            float (&wh)[R][E], uint32_t (&code)[R][E], __half2 (&meta)[R], unsigned& wabs_max, Emit emit) {
     static_assert(R == 1 || R == 2 || R == 4, "rows per step");
     const int lane = threadIdx.x & 31;
+    auto quotient_lane = [](int r) { return R == 4 ? (r >> 1) * 16 + (r & 1) * 8 : r * 16; };
     float rs[R][E];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        int mn = ordered(w[r][0]), mx = mn;
+        float fmn = INFINITY, fmx = -INFINITY;               // (compensated weights that are no numbers count for neither)
 #pragma unroll
-        for (int e = 1; e < E; ++e) { mn = min(mn, ordered(w[r][e])); mx = max(mx, ordered(w[r][e])); }
-        const float wmin = unordered(__reduce_min_sync(0xffffffffu, mn)), wmax = unordered(__reduce_max_sync(0xffffffffu, mx));
+        for (int e = 0; e < E; ++e) { fmn = fminf(fmn, w[r][e]); fmx = fmaxf(fmx, w[r][e]); }
+        const float wmin = unordered(__reduce_min_sync(0xffffffffu, ordered(fmn))), wmax = unordered(__reduce_max_sync(0xffffffffu, ordered(fmx)));
         meta[r] = group_meta(wmin, wmax, levels);
         wabs_max = max(wabs_max, __float_as_uint(fmaxf(fabsf(wmin), fabsf(wmax))));
         const float s1 = __low2float(meta[r]), lo = __high2float(meta[r]), inv = __frcp_rn(s1);
@@ -344,6 +345,7 @@ __device__ __forceinline__ void free_codes(const float (&w)[R][E], float levels,
             rs[r][e] = __fsub_rn(wc, wh[r][e]);
         }
     }
+    int numbers = 0;                                         // steps whose scale is a number, of the row this lane forms the quotient of
 #pragma unroll 1
     for (int j = 0; j < n_lv; ++j) {
         float part[R];
@@ -373,9 +375,10 @@ __device__ __forceinline__ void free_codes(const float (&w)[R][E], float levels,
         for (int off = 4; off; off >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, off));
         const float mean = USE_E ? __fdiv_rn(v, den) : __fmul_rn(v, 1.0f / (32 * E));
         const float sv = __half2float(__float2half_rn(mean));
+        if constexpr (USE_E) numbers += sv == sv;            // (a plain mean is a number whenever the residuals are)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const float sj = __shfl_sync(0xffffffffu, sv, R == 4 ? (r >> 1) * 16 + (r & 1) * 8 : r * 16);
+            const float sj = __shfl_sync(0xffffffffu, sv, quotient_lane(r));
             if (lane == 0) emit(r, j, __float2half_rn(sj));
 #pragma unroll
             for (int e = 0; e < E; ++e) residual_step(__fadd_rn(w[r][e], 0.0f), sj, wh[r][e], rs[r][e], code[r][e]);
@@ -384,10 +387,13 @@ __device__ __forceinline__ void free_codes(const float (&w)[R][E], float levels,
     const uint32_t flip = (1u << n_lv) - 1u;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        // an infinite base scale (a one-bit base whose range exceeds fp16) leaves no residual that is a number: every bit 0
-        const bool finite = !__hisinf(__low2half(meta[r]));
+        // A residual that is no number gives the bit 0.  That is every residual from the base on if the base scale is infinite (a
+        // one-bit base whose range exceeds fp16), and those after the first step whose scale is no number (a group whose
+        // weights of Eq. 5 are all zero; a step's bit is decided before its scale counts).
+        const int stand = USE_E ? __shfl_sync(0xffffffffu, numbers, quotient_lane(r)) + 1 : n_lv;
+        const uint32_t keep = __hisinf(__low2half(meta[r])) ? 0u : ~0u << max(n_lv - stand, 0);
 #pragma unroll
-        for (int e = 0; e < E; ++e) code[r][e] = finite ? code[r][e] ^ flip : 0u;
+        for (int e = 0; e < E; ++e) code[r][e] = (code[r][e] ^ flip) & keep;
     }
 }
 

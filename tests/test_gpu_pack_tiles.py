@@ -74,3 +74,24 @@ def test_pack_range_beyond_the_scale_format(B, bits, g, scale_mode):
     assert np.array_equal(np_f32(s1), q.s1) and np.array_equal(np_f32(lo), q.lo)
     if scale_mode and bits[-1] > bits[0]:
         assert np.array_equal(np_f32(B.unpack_scales(cfg, blob, rows, cols)), q.s_extra, equal_nan=True)
+
+
+@pytest.mark.parametrize("g", [32, 64, 128, 256])
+@pytest.mark.parametrize("bits", [(2, 3, 4, 8), (1, 8), (3, 5), (7, 8)])
+def test_pack_groups_without_energy(B, bits, g):
+    # columns the calibration activations never excite: where a whole group has none, the weighted mean of Eq. 5 is 0 / 0, the
+    # first residual bit stands and every later one is 0
+    from oracle import mwq
+    rows, cols = 130, 1024
+    cfg = B.Config(cols, cols, 2, 1, g, bits, scale_mode=1)
+    W = synth.normal(20, 5, (rows, cols), 0.02, "cuda")
+    energy = synth.normal(20, 6, (1, cols), 1.0, "cuda")[0].abs() + 0.1
+    energy[:256], energy[512:768], energy[900] = 0.0, 0.0, 0.0
+    blob = B.pack_mwq_calibrated(cfg, W, None, energy)
+    with np.errstate(all="ignore"):
+        q = mwq.quantize(np_f32(W), bits, g, 1, col_energy=np_f32(energy))
+    assert np.isnan(q.s_extra).any() and not np.isnan(q.s_extra).all()
+    codes, s1, lo = B.unpack_codes(cfg, blob, rows, cols, bits[-1])
+    assert np.array_equal(codes.cpu().numpy(), q.code)
+    assert np.array_equal(np_f32(s1), q.s1) and np.array_equal(np_f32(lo), q.lo)
+    assert np.array_equal(np_f32(B.unpack_scales(cfg, blob, rows, cols)), q.s_extra, equal_nan=True)
