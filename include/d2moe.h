@@ -256,9 +256,9 @@ d2moe_status d2moe_moe_forward_events(const d2moe_config* cfg, int64_t T, const 
                                       void* const* stage_events);
 
 /* Number of kernel launches one d2moe_moe_forward call enqueues for T tokens (0 on a bad config), for a
- * call that passes gate weights and widths; with more than 16 experts or at least 1024 tokens a call that
- * passes logits instead makes one launch fewer, and from 256 tokens on (with logits, or in those same cases)
- * widths chosen by the router take one more. */
+ * call that passes gate weights and widths.  With many experts or tokens the gate logits take one of them, which a
+ * call that passes logits does without; widths chosen by the router take one more in large loads (from 2048
+ * assignments on). */
 int d2moe_forward_launch_count(const d2moe_config* cfg, int64_t T, int routing_precomputed);
 
 /*

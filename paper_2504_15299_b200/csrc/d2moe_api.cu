@@ -413,9 +413,9 @@ extern "C" int d2moe_forward_launch_count(const d2moe_config* c, int64_t T, int 
         tc_plan(c, T, &pl0);
         if (pl0.decode) route -= 1;
     }
-    // more than 16 experts or many tokens: the gate logits come from a tiled kernel of their own (when the caller supplies
+    // many experts or many tokens: the gate logits come from a tiled kernel of their own (when the caller supplies
     // logits instead of gate weights that launch does not happen: the count is then one too high)
-    if (!routing_precomputed && (c->n_experts > 16 || T >= 1024) && (size_t)c->d_model * 2 * 2 <= 190 * 1024) route += 1;
+    if (!routing_precomputed && d2moe_gate_is_tiled(c->d_model, c->n_experts, T, true) && (size_t)c->d_model * 2 * 2 <= 190 * 1024) route += 1;
     if (use_tensor_path(c)) {
         TcPlan pl;
         tc_plan(c, T, &pl);

@@ -200,6 +200,18 @@ static inline bool d2moe_group_is_mid(long long A, long long n_keys) {
     return A <= 12288 && n_keys <= 2048 && n_keys * ((A + 31) / 32) <= 6144;
 }
 
+// Gate logits from the tiled kernel in a launch of its own, or from the routing kernel, whose block per token reads all gate rows in
+// batches of eight.  The tiled kernel takes 3.5 us per 1024 columns whatever it computes, a batch about 2 us at least,
+// and all batches together are bound by their reads from L2, tokens x (experts + the token's own row).  Both sides take the
+// same time at tokens x (experts + 2) = 13800 (16 x 2048), 12600 (16 x 1024), 10200 (32 x 2048); with rows of 4096 at 12000 (8
+// experts, widths supplied) and 15000 (chosen by the router), 9600 and 10500 (1 expert); where one block fills an SM at 5500 (17
+// x 8192) and 5200 (8 x 14336); with short rows, where the blocks' fixed cost counts, at 6100 (4 x 256).
+static inline bool d2moe_gate_is_tiled(long long d, long long E, long long T, bool widths_supplied) {
+    if ((E + 7) / 8 > 4) return true;
+    const long long line = d > 4096 || d <= 256 ? 6144 : (d <= 512 ? 9216 : (d <= 2048 ? 12288 : (widths_supplied ? 9216 : 10752)));
+    return T * (E + 2) > line;
+}
+
 constexpr size_t D2MOE_HIST_RUNS = 64;     // histograms the workspace holds for the grouping of large loads
 
 // Workspace carving (all offsets 256-byte aligned).

@@ -4,6 +4,8 @@
 #include "tc_common.cuh"
 #include "group_block.cuh"
 
+#include <type_traits>
+
 namespace {
 
 constexpr int MAX_TOPK = 8;
@@ -348,20 +350,24 @@ __device__ __forceinline__ void dots_halfwarp(const uint32_t* x, const uint32_t*
     }
 }
 
-// Gate logits as a tiled product: a block takes 16 tokens x 8 experts, a half-warp forms 4 x 4 of them in registers (same lane
-// layout and order as above), columns stream through shared memory 256 at a time, double buffered (so that nine blocks share an SM).  Bound: fp32 issue (a
-// multiply-add, half a conversion and a quarter of a shared load per product).
-// 1500 tokens x 64 experts x 2048: 62 us before (one dot per warp, two 2-byte shared loads per product).
-constexpr int GATE_TB = 16, GATE_EB = 8, GATE_COLS = 256, GATE_STAGES = 2;
+// Gate logits as a tiled product: a block takes 4 XT tokens x 2 WT experts, a half-warp forms XT x WT of them in registers (same
+// lane layout and order as above), columns stream through shared memory 256 at a time, STAGES chunks in flight.
+//   XT = WT = 4, two stages (nine blocks share an SM).  Bound: fp32 issue (a multiply-add, half a conversion and a quarter of a
+// shared load per product).  1500 tokens x 64 experts x 2048: 62 us before (one dot per warp, two 2-byte shared loads per product).
+//   XT = WT = 1, eight stages, for a handful of tokens: the other tile would be mostly padding, whose products a half-warp
+// would walk through all the same (56 instructions per 32 columns against 8).
+constexpr int GATE_COLS = 256;
 constexpr int GATE_PITCH = GATE_COLS / 2 + 4;           // words per row: four rows on, the other half of the banks
+template <int XT, int WT, int STAGES>
 __global__ void __launch_bounds__(128)
 gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
                    float* __restrict__ logits) {
     pdl_enter();
-    constexpr int ROWS = GATE_TB + GATE_EB;
-    __shared__ __align__(16) uint32_t sm[GATE_STAGES][ROWS][GATE_PITCH];
+    constexpr int TB = 4 * XT, ROWS = TB + 2 * WT;
+    static_assert(XT * WT <= 16, "a lane of the half-warp writes each product");
+    __shared__ __align__(16) uint32_t sm[STAGES][ROWS][GATE_PITCH];
     const int hw = threadIdx.x >> 4, p = threadIdx.x & 15;
-    const int tb = blockIdx.x * GATE_TB, eb = blockIdx.y * GATE_EB;
+    const int tb = blockIdx.x * TB, eb = blockIdx.y * (2 * WT);
     const int n_chunks = (d + GATE_COLS - 1) / GATE_COLS;
     auto stage = [&](int c) {
         if (c < n_chunks) {
@@ -370,72 +376,81 @@ gate_logits_kernel(int T, int E, int d, const __nv_bfloat16* __restrict__ x, con
                 const int r = i / (GATE_COLS / 8), k = i % (GATE_COLS / 8);
                 if (k >= n16) continue;
                 // rows past the end repeat the last one; their results are dropped
-                const __nv_bfloat16* src = r < GATE_TB ? x + (size_t)min(tb + r, T - 1) * d : gate_w + (size_t)min(eb + r - GATE_TB, E - 1) * d;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(&sm[c % GATE_STAGES][r][4 * k])), "l"(src + c0 + 8 * k) : "memory");
+                const __nv_bfloat16* src = r < TB ? x + (size_t)min(tb + r, T - 1) * d : gate_w + (size_t)min(eb + r - TB, E - 1) * d;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(&sm[c % STAGES][r][4 * k])), "l"(src + c0 + 8 * k) : "memory");
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    stage(0);
-    float acc[4][4][2];
+#pragma unroll 1
+    for (int c = 0; c < STAGES - 1; ++c) stage(c);
+    float acc[XT][WT][2];
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
+    for (int t = 0; t < XT; ++t)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[t][r][0] = acc[t][r][1] = 0.0f;
-    const int xr = (hw & 3) * 4, wr = GATE_TB + (hw >> 2) * 4;
+        for (int r = 0; r < WT; ++r) acc[t][r][0] = acc[t][r][1] = 0.0f;
+    const int xr = (hw & 3) * XT, wr = TB + (hw >> 2) * WT;
     for (int c = 0; c < n_chunks; ++c) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
         __syncthreads();                          // chunk c is there; the stage refilled next has been read
-        stage(c + 1);
-        const uint32_t (*b)[GATE_PITCH] = sm[c % GATE_STAGES];
+        stage(c + STAGES - 1);
+        const uint32_t (*b)[GATE_PITCH] = sm[c % STAGES];
         const int steps = min(GATE_COLS, d - c * GATE_COLS) / 32;
 #pragma unroll 4
         for (int i = 0; i < steps; ++i) {
-            float xv[4][2], wv[4][2];
+            float xv[XT][2], wv[WT][2];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const uint32_t v = b[xr + t][16 * i + p], u = b[wr + t][16 * i + p];
+            for (int t = 0; t < XT; ++t) {
+                const uint32_t v = b[xr + t][16 * i + p];
                 xv[t][0] = __uint_as_float(v << 16); xv[t][1] = __uint_as_float(v & 0xffff0000u);
-                wv[t][0] = __uint_as_float(u << 16); wv[t][1] = __uint_as_float(u & 0xffff0000u);
             }
 #pragma unroll
-            for (int t = 0; t < 4; ++t)
+            for (int r = 0; r < WT; ++r) {
+                const uint32_t u = b[wr + r][16 * i + p];
+                wv[r][0] = __uint_as_float(u << 16); wv[r][1] = __uint_as_float(u & 0xffff0000u);
+            }
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
+            for (int t = 0; t < XT; ++t)
+#pragma unroll
+                for (int r = 0; r < WT; ++r) {
                     acc[t][r][0] = fmaf(xv[t][0], wv[r][0], acc[t][r][0]);
                     acc[t][r][1] = fmaf(xv[t][1], wv[r][1], acc[t][r][1]);
                 }
         }
     }
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
+    for (int t = 0; t < XT; ++t)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < WT; ++r) {
 #pragma unroll
             for (int off = 8; off; off >>= 1) {
                 acc[t][r][0] += __shfl_xor_sync(0xffffffffu, acc[t][r][0], off);
                 acc[t][r][1] += __shfl_xor_sync(0xffffffffu, acc[t][r][1], off);
             }
-            const int tt = tb + xr + t, ee = eb + wr - GATE_TB + r;
-            if (p == 4 * t + r && tt < T && ee < E) logits[(size_t)tt * E + ee] = acc[t][r][0] + acc[t][r][1];
+            const int tt = tb + xr + t, ee = eb + wr - TB + r;
+            if (p == WT * t + r && tt < T && ee < E) logits[(size_t)tt * E + ee] = acc[t][r][0] + acc[t][r][1];
         }
 }
 
 // One block (8 warps) per token: the same results as route_kernel, with the token row and batches of
 // EB weight rows staged in shared memory by 16-byte loads (the pinned summation order makes a lane
 // walk a row with stride 32, which is slow straight from global memory); warp w takes row w of a batch.
-// FORCED: the widths are supplied (a kernel of its own: the code for choosing them costs such a call 1 us of instruction fetch).
-template <bool FORCED>
-__global__ void __launch_bounds__(256)
+// WIDTHS: supplied by the caller (a kernel of its own: the code for choosing them costs such a call 1 us of instruction fetch), chosen
+// from the width rows of all selected experts staged at once, or from batches of EB rows (apart from the former, whose 64
+// registers leave four blocks on an SM, this one's 48 five) or by the kernel behind it.
+enum { WIDTHS_SUPPLIED, WIDTHS_AT_ONCE, WIDTHS_BATCHED };
+template <int WIDTHS>
+__global__ void __launch_bounds__(256, WIDTHS == WIDTHS_AT_ONCE ? 4 : 5)
 route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gate_w,
                    const float* __restrict__ logits_in, const __nv_bfloat16* __restrict__ bit_w,
                    const int8_t* __restrict__ forced, RouteBufs R, int32_t* __restrict__ keys,
-                   int32_t* __restrict__ device_status, int EB, int ws_elems, int slot_pitch) {
+                   int32_t* __restrict__ device_status, int EB, int xs_elems, int ws_elems, int slot_pitch) {
     pdl_enter();
     extern __shared__ __align__(16) uint8_t rsm[];
-    // EB == 0: nothing is staged (logits and widths supplied); ws_elems: elements of the staging area behind the token row
+    // EB == 0: nothing is staged (logits and widths supplied); xs_elems, ws_elems: elements of the token row's place and of the staging
+    // area behind it
     __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(rsm);
-    __nv_bfloat16* ws = xs + (EB ? D.d : 0);
+    __nv_bfloat16* ws = xs + xs_elems;
     float* lg_s = reinterpret_cast<float*>(ws + ws_elems);               // [E]
     float* u_s = lg_s + D.E;                                             // [k * K]
     int* sel_s = reinterpret_cast<int*>(u_s + MAX_TOPK * 8);             // [k]
@@ -481,8 +496,8 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
     }
     __syncthreads();
 
-    const bool later = !FORCED && slot_pitch < 0;     // the widths are chosen by the next kernel
-    if (!FORCED && slot_pitch > 0) {   // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
+    const bool later = WIDTHS == WIDTHS_BATCHED && slot_pitch < 0;     // the widths are chosen by the next kernel
+    if constexpr (WIDTHS == WIDTHS_AT_ONCE) {   // the width rows of all selected experts at once, a half-warp per slot, four widths at a time
         for (int s = 0; s < D.k; ++s)         // (odd slots half a bank row on: the two half-warps of a warp meet no conflict)
             stage_row(ws + (size_t)s * slot_pitch, bit_w + (size_t)sel_s[s] * D.K * D.d, D.K * D.d);
         stage_wait();
@@ -511,7 +526,7 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
             }
         }
         __syncthreads();
-    } else if (!FORCED && !later) {   // bit-width router logits of the selected experts: rows (slot s, width c)
+    } else if (WIDTHS == WIDTHS_BATCHED && !later) {   // bit-width router logits of the selected experts: rows (slot s, width c)
         const int n_rows = D.k * D.K;
         for (int rb = 0; rb < n_rows; rb += EB) {
             const int n = min(EB, n_rows - rb);
@@ -535,7 +550,7 @@ route_block_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_bf
             if (s < D.k) {
                 const int a = t * D.k + s;
                 int kk = 0;
-                if (FORCED) {
+                if (WIDTHS == WIDTHS_SUPPLIED) {
                     kk = forced[a];
                     if (kk < 0 || kk >= D.K) {
                         if (device_status) atomicOr(device_status, D2MOE_DEV_BAD_INDEX);
@@ -571,38 +586,58 @@ cudaError_t launch_route(const MoeDims& D, const __nv_bfloat16* x, const __nv_bf
     int EB = row_bytes + tail_bytes < budget ? (int)((budget - row_bytes - tail_bytes) / row_bytes) : 0;
     if (EB > 8) EB = 8;
     if (EB >= 1 && D.d % 8 == 0) {
-        // Many experts or many tokens: gate logits by the tiled kernel first, then route from those logits.  (Below that a block per
-        // token reads the few gate rows itself: one launch less.)
-        // 16 experts and fewer: from 1024 tokens on (8 experts x 4096: 22 us either way there).
-        if (!logits_in && logits_ws && (D.E > 16 || D.T >= 1024)) {
-            dim3 grid((D.T + GATE_TB - 1) / GATE_TB, (D.E + GATE_EB - 1) / GATE_EB);
-            launch_chained(gate_logits_kernel, dim3(grid), dim3(128), 0, st, D.T, D.E, D.d, x, gate_w, logits_ws);
+        if (!logits_in && logits_ws && d2moe_gate_is_tiled(D.d, D.E, D.T, forced != nullptr)) {
+            const bool few = D.T <= 8;
+            dim3 grid(few ? (D.T + 3) / 4 : (D.T + 15) / 16, few ? (D.E + 1) / 2 : (D.E + 7) / 8);
+            launch_chained(few ? gate_logits_kernel<1, 1, 8> : gate_logits_kernel<4, 4, 2>, dim3(grid), dim3(128), 0, st, D.T, D.E, D.d, x, gate_w, logits_ws);
             logits_in = logits_ws;
             gate_w = nullptr;
         }
-        // staging area: EB gate rows (or width rows, batch by batch), or the width rows of all selected experts if they fit in half
-        // of what an SM has
+        // staging area: EB gate rows (or width rows, batch by batch), or the width rows of all selected experts
         if (logits_in && forced) EB = 0;
-        // many tokens with their logits at hand: one warp per token selects, the widths are chosen by a kernel of their own
-        const bool later = logits_in && !forced && D.T >= 256;
+        const size_t slots_bytes = (size_t)D.k * ((size_t)D.K * row_bytes + 64);
+        const bool fits = slots_bytes + row_bytes + tail_bytes <= 110 * 1024;                  // half of what an SM has
+        // Many pairs of token and expert with the logits at hand: one warp per token selects, the widths are chosen by a kernel of
+        // their own.  Its chain of d / 32 loads takes 29 us at d = 4096 whatever the number of pairs, which the staged
+        // forms reach at 3000 pairs (8 experts x 4096, top-2: 1024 tokens 29 staged, 36 so; 2048 tokens 47, 39), 2300 where the rows
+        // are staged batch by batch (17 experts x 8192, 6 widths).
+        const bool later = logits_in && !forced && D.A >= (fits ? 2560 : 2048);
         if (later) EB = 0;
         int slot_pitch = later ? -1 : 0;
-        if (!forced && !later && (size_t)D.k * ((size_t)D.K * row_bytes + 64) + row_bytes + tail_bytes <= 110 * 1024) slot_pitch = D.K * D.d + 32;
+        if (!forced && !later && fits) {
+            // All width rows at once need one trip to memory, batches of EB several; but they may leave fewer blocks on an SM.
+            const int rows = D.k * D.K, sms = device_sm_count();
+            auto resident = [&](size_t area) { const long long n = 228 * 1024 / (long long)(row_bytes + area + tail_bytes + 1024); return (int)(n < 8 ? n : 8); };
+            const int all = resident(!logits_in && slots_bytes < EB * row_bytes ? EB * row_bytes : slots_bytes), batched = resident(EB * row_bytes);
+            // 4 rows and fewer behind the gate's rows: the batch is one as well, and a warp per row is faster than half a one
+            // (dense layer of 4096, 2048 tokens: 44 against 49 us).  More rows than a batch: all at once while the tokens are one wave of
+            // blocks, beyond that if the trips saved outweigh the blocks lost (64 experts x 2048, top-6, 3 widths: 256 tokens 19
+            // against 23, 768 tokens 39 against 37; 16 x 1024, top-4, 4 widths: 768 tokens 19 against 30).
+            const bool at_once = rows <= EB ? logits_in || rows > 4
+                                            : D.T <= (long long)sms * all || (rows + EB - 1) / EB * all > batched;
+            if (at_once) slot_pitch = D.K * D.d + 32;
+        }
         size_t ws_elems = !EB ? 0 : slot_pitch > 0 ? (size_t)D.k * slot_pitch : (size_t)EB * D.d;
         if (EB && !logits_in && ws_elems < (size_t)EB * D.d) ws_elems = (size_t)EB * D.d;
         const size_t smem = (EB ? row_bytes : 0) + 2 * ws_elems + tail_bytes;
-        cudaError_t e = forced ? ensure_dynamic_smem<&route_block_kernel<true>>((int)smem) : ensure_dynamic_smem<&route_block_kernel<false>>((int)smem);
-        if (e != cudaSuccess) return e;
         // logits and widths both supplied: no dot products, one warp per token does the selection
         const int threads = !EB ? 32 : (logits_in && slot_pitch > 0) ? 128 : 256;
-        launch_chained(forced ? route_block_kernel<true> : route_block_kernel<false>, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB,
-                       (int)ws_elems, slot_pitch);
+        auto launch = [&](auto widths) -> cudaError_t {
+            constexpr auto kern = &route_block_kernel<decltype(widths)::value>;
+            cudaError_t e = ensure_dynamic_smem<kern>((int)smem);
+            if (e != cudaSuccess) return e;
+            launch_chained(kern, dim3(D.T), dim3(threads), smem, st, D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status, EB,
+                           EB ? D.d : 0, (int)ws_elems, slot_pitch);
+            return cudaSuccess;
+        };
+        const cudaError_t e = forced ? launch(std::integral_constant<int, WIDTHS_SUPPLIED>{})
+                            : slot_pitch > 0 ? launch(std::integral_constant<int, WIDTHS_AT_ONCE>{}) : launch(std::integral_constant<int, WIDTHS_BATCHED>{});
+        if (e != cudaSuccess) return e;
         if (later) launch_chained(width_router_kernel, dim3((D.A + 15) / 16), dim3(128), 0, st, D, x, bit_w, R, keys_ws);
     } else
     launch_chained(route_kernel, dim3((D.T + warps_per_block - 1) / warps_per_block), dim3(warps_per_block * 32), 0, st, 
         D, x, gate_w, logits_in, bit_w, forced, R, keys_ws, device_status);
-    // few assignments and keys: histogram, scan and scatter in one single-block launch (beyond about a
-    // thousand warp walks the three grid-wide kernels are faster: 39 vs 10 us at 192 keys x 1536 assignments)
+    // few assignments and keys: histogram, scan and scatter in one single-block launch
     const bool small = d2moe_group_is_small(D.A, n_keys);
     // the caller runs the single-block grouping in front of its next kernel (one launch instead of two)
     if ((small || d2moe_group_is_sortable(D.A, n_keys)) && defer_small_group) { *defer_small_group = true; return cudaGetLastError(); }

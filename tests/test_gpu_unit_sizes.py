@@ -94,3 +94,31 @@ def test_routing_of_large_batches_matches_the_oracle(B, T, E, k, d, forced):
     assert np.array_equal(r.inv_perm.cpu().numpy(), ref.grouping.inv_perm)
     assert np.array_equal(r.group_off.cpu().numpy(), ref.grouping.group_off)
     assert np.allclose(r.topk_w.cpu().numpy(), ref.topk_w, rtol=1e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("T,E,k,K,d", [(1, 40, 3, 3, 288), (5, 64, 6, 3, 2048), (8, 33, 2, 4, 320), (9, 33, 2, 4, 320),     # few tokens, many experts
+                                       (682, 16, 2, 4, 1024), (683, 16, 2, 4, 1024), (922, 8, 2, 4, 2080),                  # gate rows by the block or tiled
+                                       (300, 1, 1, 4, 512), (300, 1, 1, 8, 512),                                           # rows behind the gate's: one batch
+                                       (700, 12, 6, 3, 2048), (150, 32, 6, 3, 2048),                                       # more rows than a batch
+                                       (1279, 4, 2, 3, 64), (1280, 4, 2, 3, 64), (1023, 9, 2, 6, 8192), (1024, 9, 2, 6, 8192)])   # widths by a kernel of their own
+@pytest.mark.parametrize("source", ["weights", "logits", "weights, no workspace"])
+def test_routing_on_both_sides_of_every_line(B, T, E, k, K, d, source):
+    from oracle import routing
+    bits = tuple(range(9 - K, 9))
+    cfg = B.Config(d, 128, E, k, 32, bits)
+    x = synth.bf16_exact(synth.normal(34, T, (T, d), 1.0, "cuda"))
+    gw = synth.bf16_exact(synth.normal(34, 1, (E, d), 0.05, "cuda"))
+    bw = synth.bf16_exact(synth.normal(34, 2, (E, K, d), 0.05, "cuda"))
+    fb = synth.categorical(34, 3, (T, k), [1.0 / K] * K, "cuda")
+    gate = {"logits": synth.normal(34, 4, (T, E), 1.0, "cuda")} if source == "logits" else {"gate_w": gw}
+    call = B.route_static_scratch if source.endswith("workspace") else B.route
+    for widths in ({"bit_w": bw}, {"forced_bit_idx": fb}):
+        r = call(cfg, x, **gate, **widths)
+        torch.cuda.synchronize()
+        ref = routing.route(np_f32(x), E=E, K=K, top_k=k, renormalize=bool(cfg.renormalize),
+                            **{n: (np_f32(v) if n != "forced_bit_idx" else v.cpu().numpy()) for n, v in {**gate, **widths}.items()})
+        assert int(r.device_status.item()) == 0
+        assert np.array_equal(r.topk_idx.cpu().numpy(), ref.topk_idx)
+        assert np.array_equal(r.bit_idx.cpu().numpy(), ref.bit_idx)
+        assert np.array_equal(r.perm.cpu().numpy(), ref.grouping.perm)
+        assert np.array_equal(r.group_off.cpu().numpy(), ref.grouping.group_off)
