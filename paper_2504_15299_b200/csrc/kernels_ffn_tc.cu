@@ -983,7 +983,11 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
         // 170: - / 1137 / 1052; 64 experts of F 1408: 150 - / 532 / 568, 169 - / 604 / 607, 178 - / 651 / 630.  With free
         // scales two operand tiles a warpgroup are too few (75: 1080 / 1278 / 1223, 100: 1283 / 1296 / 1240, 150: 1604 /
         // 1340 / 1267): units of 128 or of 320.
-        pl->n_cap = avg <= 96 ? 128 : (avg <= 160 && c->scale_mode == 0 ? 192 : 320);
+        // The list {2,3,4,8} at group size 128 has a large-unit kernel without a loop over fields and four pieces to pad (30 columns on
+        // average): there 192 columns pay up to 152 tokens (d 1024, F 2048, 8 experts: 150: 92 / 94 us with 192 / 320, 160: 106 /
+        // 96; Mixtral shape 150: 1012 / 1066, 160: 1115 / 1077; 16 experts of F 1408: 142: 134 / 136, 154: 144 / 138).
+        const bool straight = c->group_size == 128 && c->n_bits == 4 && c->bits[0] == 2 && c->bits[1] == 3 && c->bits[2] == 4 && c->bits[3] == 8;
+        pl->n_cap = avg <= 96 ? 128 : (avg <= (straight ? 152 : 160) && c->scale_mode == 0 ? 192 : 320);
         pl->rows = pl->n_cap <= 192 ? 1 : 0;
     }
     const long long n_pieces = pl->decode ? (long long)c->n_experts + c->n_shared

@@ -71,6 +71,32 @@ def test_base_width_stored_as_two_fields(B, bits, scale_mode):
             assert err <= 1e-2, (T, cfg.kernel_path, err)
 
 
+@pytest.mark.parametrize("scale_mode", [0, 1])
+@pytest.mark.parametrize("bits", [(2, 3, 4, 8), (2, 4, 8), (4, 8)])
+def test_long_items_and_many_of_them(B, bits, scale_mode):
+    # Items of 32 K-groups, several per CTA (512 of gate/up and 256 or more of down per wave of units): the rings wrap many times,
+    # the accumulator and the queue are handed over between items.  Average loads on both sides of every unit width (60 |
+    # 96 | 97 | 120 | 152 | 153 | 160 | 161 tokens per expert, two experts with more, so that some units overflow), against
+    # the CUDA-core path on the same packed weights: 1e-2 of the row's largest output, the bound of the sweep above.
+    d, F, E, k, g = 4096, 4096, 8, 2, 128
+    cfg_tc, cfg_cc = (B.Config(d, F, E, k, g, bits, scale_mode=scale_mode, kernel_path=p) for p in (0, 1))
+    blobs = [B.pack_mwq(cfg_tc, synth.normal(35, 3 * e + m, (F, d) if m < 2 else (d, F), 0.02, "cuda"))
+             for e in range(E) for m in range(3)]
+    for avg in (60, 96, 97, 120, 152, 153, 160, 161):
+        T = avg * E // k
+        x = synth.bf16_exact(synth.normal(35, 1000 + T, (T, d), 1.0, "cuda"))
+        logits = synth.normal(35, 2000 + T, (T, E), 1.0, "cuda") + torch.tensor([0.6, 0.6, 0, 0, 0, 0, -0.5, -0.5], device="cuda")
+        fb = synth.categorical(35, 3000 + T, (T, k), [1.0 / len(bits)] * len(bits), "cuda")
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        y1, y1b = (B.moe_forward(cfg_tc, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st) for _ in range(2))
+        y2 = B.moe_forward(cfg_cc, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st).float()
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        assert torch.equal(y1.view(torch.int16), y1b.view(torch.int16)), ("rerun differs", avg)
+        err = float(((y1.float() - y2).abs().amax(dim=1) / y2.abs().amax(dim=1)).max())
+        assert err <= 1e-2, (avg, err)
+
+
 @pytest.mark.parametrize("T,E,k,d", [(255, 20, 3, 192), (257, 20, 3, 192),      # tiled gate logits (E > 16), width router (T >= 256)
                                      (1023, 5, 2, 320), (1029, 5, 2, 320),      # tiled gate logits from 1024 tokens
                                      (6149, 8, 2, 64), (1100, 64, 6, 64)])      # grouping over the grid: many assignments, many keys
