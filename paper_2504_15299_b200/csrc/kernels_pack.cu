@@ -461,7 +461,7 @@ pack_free_kernel(PackLayout L, const float* __restrict__ W, uint8_t* __restrict_
 // one ascending pass with the sums in registers, quantizes the group, and leaves the group's E in W's own columns, where
 // only this warp reads it again.  Nothing is written twice and no group waits for a launch.  (One pass over all later
 // columns per group instead reads and writes the whole matrix once per group and starts 2 n_groups kernels.)
-// The panel H^c[0..b, b..b+g) streams through shared memory in chunks of CAL_KC rows (double buffered, cp.async), the
+// The panel H^c[0..b, b..b+g) streams through shared memory in chunks of CAL_KC rows (two or three of them, cp.async), the
 // warp's E chunk is transposed into shared memory.
 // Bound: fp32 instruction issue, two instructions per (weight, earlier column): 6.4 ms for 14336 x 4096.
 // Measured there (one B200): 9.2 ms; one pass over all later columns per group, two launches each, took 64.8 ms.
@@ -472,6 +472,11 @@ constexpr int CAL_KC = 32;
 template <int GS, int R>
 struct CalShape {
     static constexpr int E = GS / 32;                                      // columns per lane
+    // With one or two rows a warp (few rows in all) a scheduler has a warp or two and the copies are what a chunk waits for: three
+    // chunks in flight and all loads of a chunk's products ahead of them.  (256 x 4096, group size 128: 1970 us with two
+    // chunks and four products unrolled, now 1420; 128 x 14336: 23.2 -> 16.7 ms.)
+    static constexpr int STAGES = R >= 4 ? 2 : 3;
+    static constexpr int UNROLL = R == 1 ? 32 : (R == 2 ? 16 : 4);
     // floats per warp: the E chunk [CAL_KC][R], the finished rows [R][GS], the cells of one row
     static constexpr int WARP_FLOATS = CAL_KC * R + R * GS + GS / 4;
 };
@@ -482,10 +487,11 @@ pack_calibrated_kernel(PackLayout L, float* W, const float* __restrict__ hc, con
                        uint8_t* __restrict__ packed, int n_warp_tiles, float one) {
     using C = CalShape<GS, R>;
     constexpr int E = C::E;
+    constexpr int STAGES = C::STAGES, UNROLL = C::UNROLL;
     extern __shared__ __align__(16) uint8_t smem[];
-    float* hs = reinterpret_cast<float*>(smem);                            // [2][CAL_KC][GS]
+    float* hs = reinterpret_cast<float*>(smem);                            // [STAGES][CAL_KC][GS]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
-    float* es = hs + 2 * CAL_KC * GS + warp * C::WARP_FLOATS;
+    float* es = hs + STAGES * CAL_KC * GS + warp * C::WARP_FLOATS;
     float* rows_s = es + CAL_KC * R;
     uint32_t* cs = reinterpret_cast<uint32_t*>(rows_s + R * GS);
     const float levels = (float)((1 << L.b1) - 1);
@@ -508,10 +514,13 @@ pack_calibrated_kernel(PackLayout L, float* W, const float* __restrict__ hc, con
             for (int r = 0; r < R; ++r)
 #pragma unroll
                 for (int e = 0; e < E; ++e) w[r][e] = mine && row0 + r < L.rows ? W[(row0 + r) * (long long)L.cols + b + col(e)] : 0.0f;
-            auto stage = [&](int k0, int buf) {                            // rows k0 .. k0 + CAL_KC of the panel
-                const uint32_t dst = smem_u32(hs + buf * CAL_KC * GS);
+            int fill = 0, drain = 0;                                       // stages the next chunk goes to and the next one read is in
+            auto stage = [&](int k0) {                                     // rows k0 .. k0 + CAL_KC of the panel, if it has them
+                const uint32_t dst = smem_u32(hs + fill * CAL_KC * GS);
+                if (++fill == STAGES) fill = 0;
                 const float* src = hc + (long long)k0 * L.cols + b;
-                if (hc_aligned) {
+                if (k0 >= b) {
+                } else if (hc_aligned) {
                     for (int i = threadIdx.x; i < CAL_KC * GS / 4; i += blockDim.x)
                         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * i), "l"(src + (long long)(i / (GS / 4)) * L.cols + 4 * (i % (GS / 4))) : "memory");
                 } else {
@@ -525,17 +534,21 @@ pack_calibrated_kernel(PackLayout L, float* W, const float* __restrict__ hc, con
 #pragma unroll
                 for (int r = 0; r < R; ++r) ev[r] = mine && row0 + r < L.rows ? W[(row0 + r) * (long long)L.cols + k0 + lane] : 0.0f;
             };
-            if (b > 0) { stage(0, 0); load_e(0); }
-            for (int k0 = 0, buf = 0; k0 < b; k0 += CAL_KC, buf ^= 1) {
+#pragma unroll 1
+            for (int c = 0; c < STAGES - 1; ++c) stage(c * CAL_KC);
+            if (b > 0) load_e(0);
+            for (int k0 = 0; k0 < b; k0 += CAL_KC) {
                 __syncwarp();
 #pragma unroll
                 for (int r = 0; r < R; ++r) es[lane * R + r] = -ev[r];
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                __syncthreads();                                           // the chunk is there, the other buffer is free
-                if (k0 + CAL_KC < b) { stage(k0 + CAL_KC, buf ^ 1); load_e(k0 + CAL_KC); }
+                asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+                __syncthreads();                                           // the chunk is there, the one before it has been read
+                stage(k0 + (STAGES - 1) * CAL_KC);
+                if (k0 + CAL_KC < b) load_e(k0 + CAL_KC);
+                const float* hp = hs + drain * CAL_KC * GS;
+                if (++drain == STAGES) drain = 0;
                 if (!mine) continue;                                       // such a warp only helps with the copies
-                const float* hp = hs + buf * CAL_KC * GS;
-#pragma unroll 4
+#pragma unroll UNROLL
                 for (int k = 0; k < CAL_KC; ++k) {
                     // (-e) h rounds to -(e h), so that adding it is the subtraction of the definition.  The assembler contracts a
                     // packed product and a packed sum into one fused operation (one rounding: other bits), so the sum is
@@ -711,7 +724,7 @@ static cudaError_t launch_calibrated_gs(const PackLayout& L, float* W, const flo
     const int tiles = (L.rows_pad + R - 1) / R, max_warps = R >= 4 ? 20 : 32;
     int warps = (tiles + grid - 1) / grid;
     warps = warps < 8 ? 8 : (warps > max_warps ? max_warps : warps);      // at least eight share the panel's copies
-    const int smem = (2 * CAL_KC * GS + warps * CalShape<GS, R>::WARP_FLOATS) * 4;
+    const int smem = (CalShape<GS, R>::STAGES * CAL_KC * GS + warps * CalShape<GS, R>::WARP_FLOATS) * 4;
     cudaError_t e = ensure_dynamic_smem<&pack_calibrated_kernel<GS, R>>(smem);
     if (e != cudaSuccess) return e;
     pack_calibrated_kernel<GS, R><<<grid, 32 * warps, smem, st>>>(L, W, hc, col_energy, packed, tiles, 1.0f);
