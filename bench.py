@@ -42,6 +42,12 @@ NCU_TRAFFIC = {"mixtral_decode:T64:gate_up:auto": 1042948288, "mixtral_decode:T6
                "finegrained:T256:gate_up:auto": 462040064, "finegrained:T256:down:auto": 234176768}
 
 
+def ncu_traffic(workload, T, stage, path, scale_mode):
+    """Captured traffic of the stage's kernel, None where there is no capture.  All captures are of tied scales: with free
+    scales another kernel runs, over more bytes."""
+    return NCU_TRAFFIC.get(f"{workload}:T{T}:{stage}:{path}") if scale_mode == 0 else None
+
+
 def measured_peaks():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
@@ -406,7 +412,7 @@ class LayerBench:
         achieved = dom_bytes / (stage_ms[dom] * 1e-3) / 1e9
         rf = {"bound": "hbm", "kernel": dom_name, "achieved": achieved, "peak": peak, "unit": "GB/s",
               "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
-              "traffic": NCU_TRAFFIC.get(f"{wl.name}:T{T}:{dom_name}:{self.path_name}"),
+              "traffic": ncu_traffic(wl.name, T, dom_name, self.path_name, self.scale_mode),
               "algorithmic_bytes_per_launch": dom_bytes,
               "stage_ms": dict(zip(names, stage_ms)), "stage_samples": len(used),
               "layer": {"algorithmic_bytes": layer_bytes,

@@ -92,3 +92,19 @@ def test_gpus_flag_starts_the_replicas_itself():
     assert len(lines) == 1, out.stdout
     d = json.loads(lines[0])
     assert d["n_gpus"] == 2 and d["ms_per_step"] == 2.0 and d["value"] == pytest.approx(64 * 2 / 2.0e-3)
+
+
+def test_captured_traffic_is_that_of_the_kernel_that_ran():
+    import bench
+    from paper_2504_15299_b200 import synth
+    assert bench.ncu_traffic("mixtral_decode", 64, "gate_up", "auto", 0) == bench.NCU_TRAFFIC["mixtral_decode:T64:gate_up:auto"]
+    # free scales run another kernel over more bytes: no capture, no figure
+    assert bench.ncu_traffic("mixtral_decode", 64, "gate_up", "auto", 1) is None
+    assert bench.ncu_traffic("mixtral_decode", 63, "gate_up", "auto", 0) is None
+    for key, traffic in bench.NCU_TRAFFIC.items():
+        name, tokens, stage, _ = key.split(":")
+        wl, T = synth.WORKLOADS[name], int(tokens[1:])
+        # an expert's packed bytes are read at least once at the lowest width and not ten times over
+        rows_cols = sum(r * c for r, c in (synth.expert_matrix_shape(wl, m) for m in ((0, 1) if stage == "gate_up" else (2,))))
+        top = rows_cols * (wl.n_experts + wl.n_shared) * wl.bits[-1] / 8
+        assert top * wl.bits[0] / wl.bits[-1] * 0.9 <= traffic <= 10 * top, key
