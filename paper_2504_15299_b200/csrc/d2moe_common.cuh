@@ -28,7 +28,6 @@
 // ordinary launch.  D2MOE_NO_PDL=1 in the environment turns the attribute off (ordinary launches).
 // ------------------------------------------------------------------------------------------------
 #ifdef __CUDACC__
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() { pdl_wait(); }
 #endif

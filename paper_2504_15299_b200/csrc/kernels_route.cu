@@ -195,10 +195,11 @@ width_router_kernel(MoeDims D, const __nv_bfloat16* __restrict__ x, const __nv_b
     }
 }
 
-// Grouping of large loads: a stable counting sort over the grid.  Block b owns a contiguous run of assignments and takes it 32
-// per warp at a time; an assignment's rank among the earlier ones of its key inside the run comes from a match instruction and
-// running counts in shared memory (per warp, then summed over warps: warps own contiguous pieces of each 1024).  Pass 1 leaves
-// the ranks in inv_perm and the run's histogram in hist[b]; pass 2 adds the counts of the earlier runs and of the smaller keys.
+// Grouping of large loads: a stable counting sort over the grid.  Block b owns a contiguous run of assignments and takes it 512
+// at a time, one per thread; an assignment's rank among the earlier ones of its key inside the run comes from a match instruction
+// (inside its warp) and one array of running counts in shared memory, to which the warps add in order, one after the other.
+// Pass 1 leaves the ranks in inv_perm and the run's histogram in hist[b]; pass 2 adds the counts of the earlier runs and of the
+// smaller keys.
 // (Before: one warp per key walked all assignments, twice: 62 us for 9000 assignments on 192 keys.)
 constexpr int GS_THREADS = 512, GS_MAX_RUNS = 64;
 __global__ void __launch_bounds__(GS_THREADS)
@@ -278,8 +279,9 @@ run_place_kernel(int A, int n_keys, int run, int n_runs, const int32_t* __restri
 // Small and mid-sized loads: histogram, scan and scatter in one launch.  Every block stages all keys in shared
 // memory and counts every key itself (32 warps, a key per warp at a time), so no block waits for another;
 // block b then writes the groups of the keys b, b + grid, ...  One block for decode-sized loads, a few
-// blocks for a prefill batch of a few thousand assignments on a few dozen keys.  Same warp-per-key ballot
-// walks as the three kernels above: the same stable order.  smem: A keys + n_keys + 1 ints.
+// blocks for a prefill batch of a few thousand assignments on a few dozen keys.  A warp walks the staged keys
+// with ballots, which keeps the assignments of a key in order: the same stable order as the other kernels'.
+// smem: A keys + n_keys + 1 ints.
 __global__ void __launch_bounds__(1024)
 group_block_kernel(int A, int n_keys, const int32_t* __restrict__ keys, int32_t* __restrict__ group_off,
                  int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm) {
