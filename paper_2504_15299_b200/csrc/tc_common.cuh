@@ -234,15 +234,18 @@ struct WidthList {
     __host__ __device__ static constexpr int seg_off(int gs, int j) { int o = D2MOE_TILE_ROWS * 4; for (int i = 0; i < j; ++i) o += D2MOE_TILE_ROWS * gs * w(i) / 8; return o; }
 };
 
-// exponent S of the common factor 2^-S from the header of a packed matrix
-__device__ __forceinline__ int matrix_exponent(const uint8_t* packed) {
+// exponent S of the common factor 2^-S from the header of a packed matrix; first_pos: position of the first stored field's lowest
+// bit in the base code (a base of 5 bits is stored as 4 + 1: position 1, of 6 as 4 + 2: 2, of 7 as 4 + 2 + 1: 3)
+__device__ __forceinline__ int matrix_exponent(const uint8_t* packed, int first_pos) {
     const PackHeader* h = reinterpret_cast<const PackHeader*>(packed);
     const float s1max = __uint_as_float(h->s1_max_bits);
     const float wabs = __uint_as_float(h->wabs_max_bits) + 4.0f * s1max;
     int e1, e2;
     frexpf(s1max, &e1);            // s1max = m * 2^e1, 0.5 <= m < 1  =>  s1max <= 2^e1
     frexpf(wabs, &e2);
-    int S = e1 + 9;                // s1max * 2^(24 - S) <= 2^15
+    // the first field's multiplier, s1 2^first_pos 2^(24 - S), is at most 2^15, and 2^16 less a half-precision step (s1 is a half,
+    // 65504 at most) at position 1
+    int S = e1 + 9 + max(first_pos - 1, 0);
     if (e2 - 15 > S) S = e2 - 15;  // |tile| <= 2^15
     return S;
 }

@@ -72,6 +72,33 @@ def test_base_width_stored_as_two_fields(B, bits, scale_mode):
 
 
 @pytest.mark.parametrize("scale_mode", [0, 1])
+@pytest.mark.parametrize("g", [64, 128])
+@pytest.mark.parametrize("bits", [(6, 8), (7, 8), (6, 7, 8), (6,), (7,), (4, 5, 6, 7, 8)])
+def test_base_of_six_and_seven_bits(B, bits, g, scale_mode):
+    # The first field of such a base sits two or three bits up in its code; its multiplier has to stay in fp16's range for every
+    # mantissa of the largest scale (0.02 and 0.0399: both ends of a power of two).  Bound as above, against the oracle.
+    from oracle import moe, mwq, routing
+    d, F, E, k = 256, 384, 4, 2
+    cfg = B.Config(d, F, E, k, g, bits, scale_mode=scale_mode)
+    for sigma in (0.02, 0.0399):
+        Ws = [synth.normal(36, 3 * e + m, (F, d) if m < 2 else (d, F), sigma, "cuda") for e in range(E) for m in range(3)]
+        blobs = [B.pack_mwq(cfg, W) for W in Ws]
+        triples = [tuple(mwq.quantize(np_f32(Ws[3 * e + m]), bits, g, scale_mode) for m in range(3)) for e in range(E)]
+        for T in (10, 120, 400):
+            x = synth.bf16_exact(synth.normal(36, 1000 + T, (T, d), 1.0, "cuda"))
+            logits = synth.normal(36, 2000 + T, (T, E), 1.0, "cuda")
+            fb = synth.categorical(36, 3000 + T, (T, k), [1.0 / len(bits)] * len(bits), "cuda")
+            rt = routing.route(np_f32(x), E=E, K=len(bits), top_k=k, renormalize=True, logits=np_f32(logits),
+                               forced_bit_idx=fb.cpu().numpy())
+            ref = moe.moe_layer(np_f32(x), rt, lambda e: triples[e], bits, E)
+            st = torch.zeros(1, dtype=torch.int32, device="cuda")
+            y = np_f32(B.moe_forward(cfg, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st))
+            assert int(st.item()) == 0
+            err = max(float(np.abs(y[t] - ref[t]).max() / np.abs(ref[t]).max()) for t in range(T))
+            assert err <= 1e-2, (T, sigma, err)
+
+
+@pytest.mark.parametrize("scale_mode", [0, 1])
 @pytest.mark.parametrize("bits", [(2, 3, 4, 8), (2, 4, 8), (4, 8)])
 def test_long_items_and_many_of_them(B, bits, scale_mode):
     # Items of 32 K-groups, several per CTA (512 of gate/up and 256 or more of down per wave of units): the rings wrap many times,
