@@ -18,7 +18,8 @@
 //   * one copy of every code path: a rolled loop over the stored segments with a branch per storage width, the
 //     one-bit steps of free scales rolled as well.  The loop body must stay inside the instruction cache (about a
 //     thousand instructions); straight-line code per segment took 1.6 times as long with free scales;
-//   * the widest tile goes out of the registers as it is (its half step is part of the first addend);
+//   * the widest tile goes out of the registers as it is (its half step is part of the first addend), where that costs no
+//     precision;
 //   * one thread issues all products (299 cycles a tile next to eight busy warps, 454 with a lane elected per tile).
 //
 // What bounds it: the integer-logic and packed-half pipes that unpack the codes (LOP3, HFMA2 and HADD2 together issue some
@@ -176,8 +177,12 @@ __device__ __forceinline__ ItemInfo decode_item(const TcParams& p, int item) {
 // The kernel
 // ------------------------------------------------------------------------------------------------
 // SWS: widths of the stored segments, SWS & 15 that of the first (0: any), SWS >> 4 the sum of the widths that occur later (a
-// code path each); FREE: scale_mode 1.
-template <int GS, int SWS, bool FREE>
+// code path each); FREE: scale_mode 1; FOLD: the widest tile's last addition is part of the first addend (tied scales).  That saves
+// this tile an addition and a rounding, but the other widths' constants become differences, which fp16 rounds.  Error of a layer
+// call against 64 bits (2-norm, without / with): {2,3,4,8} 2.248e-3 / 2.203e-3, {2,4,8} 2.232 / 2.190, {3,8} 2.096 / 2.068, {4,8}
+// 2.011 / 1.991, {8} 1.946 / 1.709, but {5,6,7,8} 1.986 / 1.994, {4,5,6,7,8} 2.008 / 2.016 and {5,6,7} 1.978 / 1.986: not for a
+// base of 4 bits and more with several widths above it, where it would gain 6 %.
+template <int GS, int SWS, bool FREE, bool FOLD>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMaps maps) {
     constexpr int HALVES = GS / 64;              // 64-element K slabs of the activation tile
@@ -427,7 +432,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
             const TcUnit* u = p.units + ii.unit;
             const int e = u->e, kmax = u->kmax;
             const uint8_t* mat = p.mode == 0 ? p.P.w[3 * e + blk] : p.P.w[3 * e + 2];
-            const int S = matrix_exponent(mat, p.L.seg_shift[0] - (p.L.top - p.L.b1));
+            const int S = matrix_exponent(mat, SWS ? 0 : p.L.seg_shift[0] - (p.L.top - p.L.b1));
             const float two_mS = exp2f((float)-S);
             unsigned present = 0;
             for (int kk = 0; kk <= kmax; ++kk) present |= (u->cnt[kk] > 0 ? 1u : 0u) << kk;
@@ -479,7 +484,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
                 // code for every segment was 1.6 times slower with free scales (three in four stalls: no instruction).
                 // the widest tile's constant: half a step of its width (free scales: the sum of all steps' scales, which costs more to
                 // form in advance than it saves)
-                const float widest = FREE ? 0.0f : 0.5f * s1 * __int_as_float(seg_tab[smax].z) * two_mS;
+                const float widest = FOLD ? 0.5f * s1 * __int_as_float(seg_tab[smax].z) * two_mS : 0.0f;
                 float csum = 0.0f;                               // free scales: sum of the scales folded in so far, times 2^-S
                 int4 tb = seg_tab[0];
                 // the field's multiplier: s1 2^(position - (top - b1)) 2^-S, and for a code at bit position 0 of its lane
@@ -500,7 +505,7 @@ ffn_row_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMa
 #pragma unroll 1
                 for (int sj = 0;;) {
                     // the last field of a width's step sits at that width's unit: half a step completes the tile
-                    if (((tb.x >> 16) & 1) && ((present >> ((tb.x >> 8) & 255)) & 1u)) write_tile((FREE ? -csum : 0.5f * Ms) - widest, !FREE && sj == smax);
+                    if (((tb.x >> 16) & 1) && ((present >> ((tb.x >> 8) & 255)) & 1u)) write_tile((FREE ? -csum : 0.5f * Ms) - widest, FOLD && sj == smax);
                     if (++sj > smax) break;
                     tb = seg_tab[sj];
                     const int sw = tb.x & 255, kk = (tb.x >> 8) & 255;
@@ -673,19 +678,22 @@ cudaError_t launch_ffn_row(const d2moe_config* c, const MoeDims& D, const PackLa
             launch_chained(kern, dim3(sms), dim3(TC_THREADS), smem_bytes, st, p, mode == 0 ? maps_x : maps_h);
             return cudaSuccess;
         };
-#define TC_KERNEL(GS_, SWS_, FREE_) std::integral_constant<decltype(&ffn_row_kernel<GS_, SWS_, FREE_>), &ffn_row_kernel<GS_, SWS_, FREE_>>{}
-#define TC_LAUNCH(GS_, SWS_) (p.L.scale_mode == 1 ? launch(TC_KERNEL(GS_, SWS_, true)) : launch(TC_KERNEL(GS_, SWS_, false)))
+#define TC_KERNEL(GS_, SWS_, FREE_, FOLD_) std::integral_constant<decltype(&ffn_row_kernel<GS_, SWS_, FREE_, FOLD_>), &ffn_row_kernel<GS_, SWS_, FREE_, FOLD_>>{}
+#define TC_LAUNCH(GS_, SWS_) (p.L.scale_mode == 1 ? launch(TC_KERNEL(GS_, SWS_, true, false)) : launch(TC_KERNEL(GS_, SWS_, false, true)))
+#define TC_LAUNCH_ANY(GS_) (p.L.scale_mode == 0 && !fold ? launch(TC_KERNEL(GS_, 0, false, false)) : TC_LAUNCH(GS_, 0))
         // a kernel of their own for the lists {2,3,4,8} (base 2, steps of 1, 1, 4) and {2,4,8}: the others take one with a path for
         // every storage width.  `sws` does not say where the base ends: the list {3,8} has the same one as {2,3,4,8}, but its base
         // is the first two fields.  With tied scales that is all one; with free scales the two kernels fold every field
         // after the first bit by bit, so a base of more than one field goes to the general kernel.
         const bool one_field_base = p.L.scale_mode == 0 || p.L.last_seg[0] == 0;
+        const bool fold = p.L.b1 < 4 || p.L.n_widths < 3;
         cudaError_t e;
-        if (!one_field_base && D.g == 128) e = TC_LAUNCH(128, 0);
+        if (!one_field_base && D.g == 128) e = TC_LAUNCH_ANY(128);
         else if (D.g == 128 && sws == 0x52) e = TC_LAUNCH(128, 0x52);
         else if (D.g == 128 && sws == 0x62) e = TC_LAUNCH(128, 0x62);
-        else if (D.g == 128) e = TC_LAUNCH(128, 0);
-        else e = TC_LAUNCH(64, 0);
+        else if (D.g == 128) e = TC_LAUNCH_ANY(128);
+        else e = TC_LAUNCH_ANY(64);
+#undef TC_LAUNCH_ANY
 #undef TC_LAUNCH
 #undef TC_KERNEL
         if (e != cudaSuccess) return e;

@@ -450,7 +450,7 @@ ffn_tc_kernel(const __grid_constant__ TcParams p, const __grid_constant__ TmaMap
             const TcUnit* u = p.units + ii.unit;
             const int e = u->e, kmax = u->kmax;
             const uint8_t* mat = p.mode == 0 ? p.P.w[3 * e + blk] : p.P.w[3 * e + 2];
-            const int S = matrix_exponent(mat, p.L.seg_shift[0] - (p.L.top - p.L.b1));
+            const int S = matrix_exponent(mat, WPACK ? 0 : p.L.seg_shift[0] - (p.L.top - p.L.b1));
             const float two_mS = exp2f((float)-S);
             unsigned present = 0;
             for (int kk = 0; kk <= kmax; ++kk) present |= (u->cnt[kk] > 0 ? 1u : 0u) << kk;

@@ -98,6 +98,24 @@ def test_base_of_six_and_seven_bits(B, bits, g, scale_mode):
             assert err <= 1e-2, (T, sigma, err)
 
 
+@pytest.mark.parametrize("g", [64, 128])
+@pytest.mark.parametrize("bits,scale_mode", [((5, 6, 7, 8), 0), ((4, 5, 6, 7, 8), 0), ((4, 6, 8), 0), ((2, 3, 4, 8), 1), ((5, 6, 7, 8), 1)])
+def test_small_units_round_as_large_ones(B, bits, scale_mode, g):
+    # Where the small-unit kernel does not fold the widest tile's constant into the first addend (a base of 4 bits and more with several
+    # widths above it, for which that lost precision, and free scales) it forms the large-unit kernel's tiles bit for bit:
+    # the same tokens alone (60 and 140 per expert) and inside a batch of 200 per expert.  F is short, so no split over K.
+    d, F, E, k = 256, 384 if g == 128 else 192, 4, 2
+    cfg = B.Config(d, F, E, k, g, bits, scale_mode=scale_mode)
+    blobs = [B.pack_mwq(cfg, synth.normal(37, 3 * e + m, (F, d) if m < 2 else (d, F), 0.02, "cuda")) for e in range(E) for m in range(3)]
+    x = synth.bf16_exact(synth.normal(37, 1000, (400, d), 1.0, "cuda"))
+    logits = synth.normal(37, 2000, (400, E), 1.0, "cuda")
+    fb = synth.categorical(37, 3000, (400, k), [1.0 / len(bits)] * len(bits), "cuda")
+    y = [B.moe_forward(cfg, x[:T].contiguous(), blobs, logits=logits[:T].contiguous(), forced_bit_idx=fb[:T].contiguous())
+         for T in (120, 280, 400)]
+    for part in y[:2]:
+        assert torch.equal(part.view(torch.int16), y[2][:part.shape[0]].view(torch.int16))
+
+
 @pytest.mark.parametrize("scale_mode", [0, 1])
 @pytest.mark.parametrize("bits", [(2, 3, 4, 8), (2, 4, 8), (4, 8)])
 def test_long_items_and_many_of_them(B, bits, scale_mode):
