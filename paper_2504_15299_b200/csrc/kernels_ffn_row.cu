@@ -25,7 +25,7 @@
 // What bounds it: the latency of dependent arithmetic with two dequant warps per scheduler.  They issue in 55 % of the cycles
 // (2.19 instructions per clock and SM; logic pipe 36 %, packed-half pipe 40 %, tensor pipe 19 %, DRAM 23 % busy; 0.8 warps
 // eligible), and no third warp fits beside 168 registers a thread and a full tensor memory.  Free residual scales take
-// seven one-bit steps per code where tied ones take three fields.  Measured (layer call, before: ffn_tc_kernel with
+// seven one-bit steps per code where tied ones take three fields (with up to 40 tokens per expert ffn_step_kernel takes most of those loads).  Measured (layer call, before: ffn_tc_kernel with
 // units of 128 to 320): d 4096, F 14336, 8 experts, top-2, widths {2,3,4,8}, 333 tokens 998 -> 835 us; free scales, 64 tokens 1157 ->
 // 1022 us; 64 experts of F 1408, top-6, 1500 tokens 590 -> 537 us.
 //

@@ -1,0 +1,698 @@
+// Grouped dequant-GEMM on the 5th-generation tensor cores for decode-sized loads with free residual scales: one operand tile per
+// stored segment.
+//
+// The nested code is a sum over its segments (W_hat at a width = the base's share + the shares of the steps up to that width), and a
+// product with a sum is a sum of products: the tile of a segment holds that segment's share alone (base: lo + s1 Q; a step of w bits:
+// sum over its bits of s_l (2 bit_l - 1), its constant in the first addend) and is multiplied by the tokens of its width and of all wider
+// ones, which are the last columns of the unit.  Against one tile per width built by a running sum (ffn_row_kernel) that takes the
+// addition of a constant per tile and the 64 registers of the running sum out of the dequantization (a tile is formed and stored 16
+// registers at a time), and a share is rounded at its own magnitude instead of the weight's: the error of a layer call against 64
+// bits falls from 1.768e-3 to 1.679e-3 (d 4096, F 14336, {2,3,4,8}, 64 tokens; no list measured worse).  It costs products, the sum of the suffixes instead of
+// the columns once, which is little while a unit holds few tokens.
+//
+// The two dequant warpgroups take alternate K-groups, whole rows per thread, and share nothing: each has operand tiles, an issuing
+// thread and an accumulator of its own, and the epilogue adds the two accumulators.  With one issuer in group order a warpgroup
+// that had filled its tiles waited for the other's group (1300 us with two or three warpgroups where this takes 740).
+// A look at a barrier takes about 100 cycles even when its phase is over, so a tile's barrier is asked for ahead of the work that
+// comes before it (864 -> 795 us), and what does not need the tile (loading the words, the multipliers, the first 16 registers) is done
+// before the wait.  Units of 64 columns leave room for three tiles a warpgroup, units of 128 for two (795 -> 736 us).
+//
+// What bounds it: the dependent arithmetic of two dequant warps per scheduler (about 3.3 cycles an instruction; 1050 instructions per row
+// and group, 896 of them the AND and the packed FMA of seven steps).  Measured (layer call, ffn_row_kernel -> this kernel): d 4096, F
+// 14336, 8 experts, top-2, {2,3,4,8}: 1 token 135 -> 118 us, 8 579 -> 485, 64 1020 -> 740, 160 1057 -> 830; {2,4,8} 64 tokens 920 ->
+// 696; {5,6,7,8} 945 -> 872; 64 experts of F 1408, top-6, 256 tokens 519 -> 439.
+//
+// Warp roles (384 threads, 1 CTA per SM, all 512 TMEM columns): warps 0-3 and 4-7 the dequant warpgroups (thread = weight row =
+// TMEM lane; lanes 2i and 2i + 1 hold row i of the tile's two packed blocks, for gate/up the two rows of one hidden unit, which the
+// epilogue pairs with a shuffle), which also take alternate 16-column chunks of the epilogue; warp 8 streams packed blocks
+// (cp.async.bulk), warp 9 activation tiles (TMA, 128B swizzle, boxes of 16 to 128 rows), warps 10 and 11 issue the MMAs.  Every wait is
+// bounded: on expiry the CTA raises D2MOE_DEV_TIMEOUT, stops waiting, drains and exits.
+#include "d2moe_common.cuh"
+#include "kernels_ffn_tc.cuh"
+#include "tc_common.cuh"
+
+#include <type_traits>
+
+namespace {
+
+constexpr int NWG = 2;                 // dequant warpgroups, each with an issuer, an accumulator and operand tiles of its own
+constexpr int ST_THREADS = 128 * NWG + 128;  // and weight producer, activation producer, the MMA issuers
+constexpr int WARP_WPROD = 4 * NWG, WARP_BPROD = WARP_WPROD + 1, WARP_MMA = WARP_WPROD + 2;
+constexpr int TMEM_COLS = 512;
+constexpr int MAX_SPW = 3;
+// operand tiles (64 TMEM columns each, behind the accumulators) per warpgroup, for accumulators of CAP columns
+__host__ __device__ constexpr int tiles_per_wg(int cap) { return cap <= 64 ? 3 : 2; }
+constexpr int MAX_NSB = 4;             // activation ring depth (upper bound)
+constexpr int MAX_NSW = 8;             // weight ring depth (upper bound)
+constexpr int NSQ = 4;                 // entries of the work queue between the weight producer and the other warps
+
+struct StepParams {
+    MoeDims D;
+    PackLayout L;
+    ExpertPtrs P;
+    int mode;                 // 0: gate/up + SwiGLU -> hbuf;  1: down -> obuf
+    int n_row_tiles, n_split, groups_per_split, nsw, nsb;
+    const TcUnit* units;
+    const int* n_units;
+    int* next_item;           // work counter of this launch: starts at the grid size (item i < grid goes to CTA i)
+    __half* hbuf;             // [R, F]
+    float* obuf;              // [n_split][R, d]
+    const float* row_scale;   // [3][R]: per padded row the power-of-two factors of the activation scaling (see tc_gather_kernel)
+    long long R_alloc;
+    int32_t* status;
+    int smem_w_off, smem_bar_off;
+};
+
+// Sixteen registers (32 codes, block b of a row) of a stored segment of SW bits per code: SW words.
+template <int GS, int SW>
+__device__ __forceinline__ void load_block(uint32_t row, int b, uint32_t (&w)[SW]) {
+    constexpr int CS = GS * SW / 8 < 16 ? GS * SW / 8 : 16;
+    const int ob = 4 * SW * b;
+    const uint32_t addr = row + (uint32_t)((ob / CS) * D2MOE_TILE_ROWS * CS + ob % CS);
+    if constexpr (SW == 8) {
+        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr));
+        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "r"(addr + D2MOE_TILE_ROWS * CS));
+    } else if constexpr (SW == 4) {
+        asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr));
+    } else if constexpr (SW == 2) {
+        asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(addr));
+    } else {
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[0]) : "r"(addr));
+    }
+}
+
+// One field of every code of a block (the bits of `field`, repeated in both halves of the mask) as half pairs: v = field * mult + addend
+template <int SW>
+__device__ __forceinline__ void fma_block(const uint32_t (&w)[SW], uint32_t field, const uint32_t (&mult)[8 / SW], uint32_t c, uint32_t (&v)[16]) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        constexpr int PER = 16 / SW;                            // registers per word
+        const int e = i % PER;
+        const uint32_t src = (e & 1) ? w[i / PER] >> 8 : w[i / PER];      // pair e of the word: bytes (0,2) or (1,3), bit SW*(e/2)
+        v[i] = hfma2_bits(src & (field << ((e >> 1) * SW)), mult[e >> 1], c);
+    }
+}
+template <int SW>
+__device__ __forceinline__ void fma_block_more(const uint32_t (&w)[SW], uint32_t field, const uint32_t (&mult)[8 / SW], uint32_t (&v)[16]) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        constexpr int PER = 16 / SW;
+        const int e = i % PER;
+        const uint32_t src = (e & 1) ? w[i / PER] >> 8 : w[i / PER];
+        v[i] = hfma2_bits(src & (field << ((e >> 1) * SW)), mult[e >> 1], v[i]);
+    }
+}
+// multipliers of the fields at bit positions 0, SW, 2 SW, ... of a byte lane, from that of position 0
+template <int SW>
+__device__ __forceinline__ void field_mults(float m0, uint32_t (&mult)[8 / SW]) {
+    mult[0] = as_u32(h2dup(m0));
+    const uint32_t step = (uint32_t)(15 - SW) * 0x04000400u;            // 2^-SW, exact
+#pragma unroll
+    for (int q = 1; q < 8 / SW; ++q) mult[q] = hmul2_bits(mult[q - 1], step);
+}
+
+// The operand tile of one stored segment of one row, written to tensor memory from dst: c + m0 * (bits of the codes).
+template <int GS, int SW>
+__device__ __forceinline__ void write_segment(uint32_t row, float m0, uint32_t c, uint32_t dst) {
+    uint32_t mult[8 / SW];
+    field_mults<SW>(m0, mult);
+#pragma unroll
+    for (int b = 0; b < GS / 32; ++b) {
+        uint32_t w[SW], v[16];
+        load_block<GS, SW>(row, b, w);
+        fma_block<SW>(w, ((1u << SW) - 1u) * 0x00010001u, mult, c, v);
+        tc_st16(dst + b * 16, v);
+    }
+}
+
+// Free residual scales (scale_mode 1): a segment after the first is SW one-bit steps, each with its own scale:
+// c + sum over its bits of (2 s_l) bit_l, c = minus the sum of the scales.
+//   sc      shared address of this row's scale of the segment's lowest bit; bit t's lies t planes before
+template <int GS, int SW>
+__device__ __forceinline__ void write_bits(uint32_t row, uint32_t sc, float two_mS, uint32_t dst) {
+    uint32_t mult[SW][8 / SW];
+    float sum = 0.0f;
+#pragma unroll
+    for (int t = 0; t < SW; ++t) {
+        unsigned short raw;
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(raw) : "r"(sc - (uint32_t)(t * D2MOE_TILE_ROWS * 2)));
+        const float sl = __half2float(__ushort_as_half(raw)) * two_mS;
+        sum += sl;
+        field_mults<SW>(sl * __int_as_float((127 + 25 - t) << 23), mult[t]);       // 2 s_l 2^(24 - t)
+    }
+    const uint32_t c = as_u32(h2dup(-sum));
+#pragma unroll 1
+    for (int b = 0; b < GS / 32; ++b) {
+        uint32_t w[SW], v[16];
+        load_block<GS, SW>(row, b, w);
+        fma_block<SW>(w, 0x00010001u, mult[0], c, v);
+#pragma unroll
+        for (int t = 1; t < SW; ++t) fma_block_more<SW>(w, 0x00010001u << t, mult[t], v);
+        tc_st16(dst + b * 16, v);
+    }
+}
+
+// The same in pieces, for width lists that are known at compile time: everything that does not need the operand tile (its words, its
+// multipliers, its first block) is done before the wait for it.
+template <int GS, int SW, int NT>
+struct SegTile {
+    uint32_t w[GS / 32][SW], mult[NT][8 / SW], c;
+    __device__ __forceinline__ void load(uint32_t row) {
+#pragma unroll
+        for (int b = 0; b < GS / 32; ++b) load_block<GS, SW>(row, b, w[b]);
+    }
+    __device__ __forceinline__ void block(int b, uint32_t (&v)[16]) const {
+        if constexpr (NT == 1) {
+            fma_block<SW>(w[b], ((1u << SW) - 1u) * 0x00010001u, mult[0], c, v);
+        } else {
+            fma_block<SW>(w[b], 0x00010001u, mult[0], c, v);
+#pragma unroll
+            for (int t = 1; t < NT; ++t) fma_block_more<SW>(w[b], 0x00010001u << t, mult[t], v);
+        }
+    }
+};
+
+struct ItemInfo {
+    int unit, tile, split, g0, g1;
+};
+
+__device__ __forceinline__ ItemInfo decode_item(const StepParams& p, int item) {
+    ItemInfo it;
+    const int per_unit = p.n_row_tiles * p.n_split;
+    it.unit = item / per_unit;
+    const int rem = item - it.unit * per_unit;
+    it.tile = rem / p.n_split;
+    it.split = rem - it.tile * p.n_split;
+    it.g0 = it.split * p.groups_per_split;
+    it.g1 = min(p.L.n_groups, it.g0 + p.groups_per_split);
+    return it;
+}
+
+// WPACK: a width list whose steps are one stored segment each (nibble j: width of step j), 0: any list; CAP: columns of a unit
+template <int GS, int WPACK, int CAP>
+__global__ void __launch_bounds__(ST_THREADS, 1)
+ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ TmaMaps maps) {
+    constexpr int HALVES = GS / 64;              // 64-element K slabs of the activation tile
+    constexpr int SPW = tiles_per_wg(CAP);
+    static_assert(NWG == 2 && SPW <= MAX_SPW && NWG * (CAP + 64 * SPW) <= 512, "tensor memory");
+    extern __shared__ uint8_t smem_raw[];
+    // shared layout (from a 1024-byte boundary, which the 128B-swizzled operand tiles need):
+    // [activation ring: nsb x CAP*GS*2] [weight ring: nsw x 2 blocks] [barriers]
+    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t smem_base = smem_u32(smem);
+    constexpr uint32_t b_slot_bytes = (uint32_t)CAP * GS * 2;
+    const uint32_t w_slot_bytes = 2u * (uint32_t)p.L.block_bytes;
+    const uint32_t bbuf = smem_base;
+    const uint32_t wbuf = smem_base + p.smem_w_off;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.smem_bar_off);
+    const uint32_t bar0 = smem_u32(bars);
+    auto W_FULL = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+    auto W_EMPTY = [&](int i) { return bar0 + 8u * (uint32_t)(MAX_NSW + i); };
+    auto B_FULL = [&](int i) { return bar0 + 8u * (uint32_t)(2 * MAX_NSW + i); };
+    auto B_EMPTY = [&](int i) { return bar0 + 8u * (uint32_t)(2 * MAX_NSW + MAX_NSB + i); };
+    constexpr int BAR_A = 2 * MAX_NSW + 2 * MAX_NSB;
+    auto A_FULL = [&](uint32_t i) { return bar0 + 8u * (BAR_A + i); };
+    auto A_EMPTY = [&](uint32_t i) { return bar0 + 8u * (BAR_A + NWG * MAX_SPW + i); };
+    constexpr int BAR_D = BAR_A + 2 * NWG * MAX_SPW;
+    auto D_FULL = [&](uint32_t i) { return bar0 + 8u * (BAR_D + i); };
+    auto D_EMPTY = [&](uint32_t i) { return bar0 + 8u * (BAR_D + NWG + i); };
+    constexpr int BAR_SQ = BAR_D + 2 * NWG;
+    auto SQ_FULL = [&](uint32_t i) { return bar0 + 8u * (BAR_SQ + i); };
+    auto SQ_EMPTY = [&](uint32_t i) { return bar0 + 8u * (BAR_SQ + NSQ + i); };
+    constexpr int BAR_END = BAR_SQ + 2 * NSQ;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + BAR_END);
+    // work queue: the weight producer takes work items from a global counter and publishes them to the other warps, so that CTAs
+    // that drew cheap items take more of them
+    volatile int* sq_item = reinterpret_cast<volatile int*>(bars + BAR_END + 1);
+    static_assert(8 * (BAR_END + 1) + 4 * NSQ <= 496, "barrier block");
+    // tail of the 512-byte barrier block, where the waits look for them: device-status pointer (496), abort flag (504)
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(reinterpret_cast<uint8_t*>(bars) + 504);
+    // behind it, per stored segment: {storage width | width index << 8, byte offset, bits of 2^(position - (top - b1)), scale_mode 1:
+    // byte offset of the scale of the field's lowest bit}
+    int4* seg_tab = reinterpret_cast<int4*>(reinterpret_cast<uint8_t*>(bars) + 512);
+
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < MAX_NSW; ++i) { mbar_init(W_FULL(i), 1); mbar_init(W_EMPTY(i), 4); }
+        for (int i = 0; i < MAX_NSB; ++i) { mbar_init(B_FULL(i), 1); mbar_init(B_EMPTY(i), 1); }
+        for (int i = 0; i < NWG * SPW; ++i) { mbar_init(A_FULL(i), 4); mbar_init(A_EMPTY(i), 1); }
+        for (int i = 0; i < NWG; ++i) { mbar_init(D_FULL(i), 1); mbar_init(D_EMPTY(i), 4 * NWG); }
+        for (int i = 0; i < NSQ; ++i) { mbar_init(SQ_FULL(i), 1); mbar_init(SQ_EMPTY(i), 1 + NWG + 4 * NWG); }
+        *abort_flag = 0;
+        *reinterpret_cast<int32_t**>(reinterpret_cast<uint8_t*>(bars) + 496) = status_or_sink(p.status);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (threadIdx.x < 8) {
+        const int j = threadIdx.x;
+        const int kk = p.L.seg_kk[j];
+        const int e = p.L.seg_shift[j] - (p.L.top - p.L.b1);
+        const int sc_t0 = p.L.w_sc_off[kk] + ((p.L.top - p.L.b1 - 1 - p.L.seg_shift[j]) - p.L.w_lv0[kk]) * D2MOE_TILE_ROWS * 2;
+        seg_tab[j] = make_int4(p.L.seg_sw[j] | (kk << 8), p.L.seg_off[j], (127 + e) << 23, sc_t0);
+    }
+    if (warp == WARP_MMA) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = (uint32_t)uniform((int)*tmem_slot);
+    const uint32_t d_tmem = tmem_base;                       // NWG accumulators of CAP columns
+    const uint32_t a_tmem = tmem_base + NWG * CAP;           // NWG * SPW tiles, 64 columns apart
+
+    // set-up done (barriers, TMEM): from here on the kernel reads what the kernels before it wrote
+    pdl_wait();
+    const int n_units = uniform(*p.n_units);
+    const int total_items = n_units * p.n_row_tiles * p.n_split;
+    const int nsw = p.nsw;
+    // next work item of a consumer: queue entry qi (one arrival per warp, or per thread for a single-thread role)
+    auto pop = [&](uint32_t qi, bool whole_warp) -> int {
+        const uint32_t q = qi & (NSQ - 1);
+        mbar_wait_blk(SQ_FULL(q), (qi / NSQ) & 1u);
+        const int item = sq_item[q];
+        if (whole_warp) __syncwarp();
+        if (!whole_warp || lane == 0) mbar_arrive(SQ_EMPTY(q));
+        return item;
+    };
+
+    if (warp == WARP_WPROD) {
+        // ---------------- weight producer ----------------
+        if (lane == 0) {
+            uint32_t it = 0, wph = 0;
+            int ws = 0;
+            int item = blockIdx.x;
+            for (uint32_t qi = 0;; ++qi) {
+                const uint32_t q = qi & (NSQ - 1);
+                mbar_wait_blk(SQ_EMPTY(q), ((qi / NSQ) & 1u) ^ 1u);
+                if (item >= total_items) item = -1;                    // the end mark
+                sq_item[q] = item;
+                mbar_arrive(SQ_FULL(q));
+                if (item < 0) break;
+                const int next = atomicAdd(p.next_item, 1);            // in flight while this item's blocks are issued
+                const ItemInfo ii = decode_item(p, item);
+                const TcUnit* u = p.units + ii.unit;
+                const int e = u->e, kmax = u->kmax;
+                const uint32_t bytes = (uint32_t)d2moe_prefix_bytes(p.L, kmax);
+                const uint8_t *m0, *m1;
+                int rt0, rt1;
+                if (p.mode == 0) { m0 = p.P.w[3 * e + 0]; m1 = p.P.w[3 * e + 1]; rt0 = rt1 = ii.tile; }
+                else { m0 = m1 = p.P.w[3 * e + 2]; rt0 = 2 * ii.tile; rt1 = 2 * ii.tile + 1; }
+                for (int G = ii.g0; G < ii.g1; ++G, ++it) {
+                    const int s = ws;                                  // ring slot and parity advance by addition
+                    mbar_wait_blk(W_EMPTY(s), wph ^ 1u);
+                    if (*abort_flag) break;                            // nothing more is copied
+                    if (++ws == nsw) { ws = 0; wph ^= 1u; }
+                    mbar_expect_tx(W_FULL(s), 2 * bytes);
+                    const uint32_t dst = wbuf + s * w_slot_bytes;
+                    bulk_g2s(dst, m0 + d2moe_block_offset(p.L, rt0, G), bytes, W_FULL(s));
+                    bulk_g2s(dst + p.L.block_bytes, m1 + d2moe_block_offset(p.L, rt1, G), bytes, W_FULL(s));
+                }
+                item = next;
+            }
+            // drain: every copy issued must have landed before the CTA may exit
+            for (int s = 0; s < nsw && s < (int)it; ++s) {
+                const uint32_t last = it - 1 - (it - 1 - s) % nsw;   // last iteration that used slot s
+                mbar_wait(W_FULL(s), (last / nsw) & 1, abort_flag, p.status, true);
+            }
+        }
+    } else if (warp == WARP_BPROD) {
+        // ---------------- activation producer ----------------
+        if (lane == 0) {
+            uint32_t it = 0, bph = 0;
+            int bs = 0;
+            for (uint32_t qi = 0;; ++qi) {
+                const int item = pop(qi, false);
+                if (item < 0) break;
+                const ItemInfo ii = decode_item(p, item);
+                const TcUnit* u = p.units + ii.unit;
+                const int ncols = u->ncols;                       // multiple of 16, <= CAP
+                const int row0 = u->row0;                         // read once: the copies below are issued back to back
+                const uint32_t bytes = (uint32_t)ncols * 128u * HALVES;
+                for (int G = ii.g0; G < ii.g1; ++G, ++it) {
+                    const int s = bs;
+                    mbar_wait_blk(B_EMPTY(s), bph ^ 1u);
+                    if (*abort_flag) break;
+                    if (++bs == p.nsb) { bs = 0; bph ^= 1u; }
+                    mbar_expect_tx(B_FULL(s), bytes);
+                    const uint32_t dst = bbuf + s * b_slot_bytes;
+                    // the rows of the unit as boxes of 128, 64, 32, 16 rows (largest first)
+                    int r = 0;
+                    for (int mi = 3; mi >= 0; --mi) {
+                        const int box = 16 << mi;
+                        while (ncols - r >= box) {
+#pragma unroll
+                            for (int h = 0; h < HALVES; ++h)
+                                tma_load_2d(dst + h * (uint32_t)CAP * 128u + (uint32_t)r * 128u, &maps.m[mi],
+                                            G * GS + h * 64, row0 + r, B_FULL(s));
+                            r += box;
+                        }
+                    }
+                }
+            }
+            for (int s = 0; s < p.nsb && s < (int)it; ++s) {
+                const uint32_t last = it - 1 - (it - 1 - s) % p.nsb;
+                mbar_wait(B_FULL(s), (last / p.nsb) & 1, abort_flag, p.status, true);
+            }
+        }
+    } else if (warp >= WARP_MMA) {
+        // ---------------- MMA issuers: one thread for each dequant warpgroup ----------------
+        // An issuer is a serial resource (one hand-off per tile), so everything an MMA needs is a register
+        // add away: per item the pieces' instruction descriptors, D columns and row offsets; per stage the low word of the shared-memory
+        // descriptor (its high word is a constant).  A look at a barrier takes 100 cycles even when its phase is over, so each tile's is
+        // asked for before the products of the one before it are issued.
+        constexpr uint32_t DESC_HI = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);
+        constexpr uint32_t SLAB_STEP = (uint32_t)CAP * 8u;        // second 64-column slab of a stage, in 16-byte units
+        if (elect_one()) {
+        const uint32_t wg = (uint32_t)(warp - WARP_MMA);
+        uint32_t bph = 0, ic = 0, sl = 0, slph = 0;               // sl: the warpgroup's next operand tile
+        int bs = (int)wg, turn = (int)wg;                         // turn: groups until the warpgroup's next one
+        bool ready = false;                                       // that tile has been seen full
+        for (uint32_t qi = 0;; ++qi, ++ic) {
+            const int item = pop(qi, false);
+            if (item < 0) break;
+            const ItemInfo ii = decode_item(p, item);
+            const TcUnit* u = p.units + ii.unit;
+            const int kmax = u->kmax, ncols = u->ncols;
+            uint32_t id0[8], dc[8], bo[8];                        // per stored segment: descriptor, D column, B rows / 16 B
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                // its tile is multiplied by the tokens of its width and of the wider ones
+                int col0 = ncols;
+                if (j < p.L.n_seg) for (int kk = kmax; kk >= p.L.seg_kk[j]; --kk) col0 = u->cnt[kk] > 0 ? u->col0[kk] : col0;
+                id0[j] = col0 < ncols ? instr_desc_f16(ncols - col0) : 0u;
+                dc[j] = d_tmem + wg * CAP + col0;
+                bo[j] = (uint32_t)col0 * 8u;
+            }
+            mbar_wait_blk(D_EMPTY(wg), (ic & 1) ^ 1);
+            tc_fence_after();
+            uint32_t accum = 0;
+            for (int G = ii.g0; G < ii.g1; ++G) {
+                if (turn != 0) { --turn; continue; }                 // another warpgroup's
+                turn = NWG - 1;
+                const int s = bs;
+                mbar_wait_blk(B_FULL(s), bph);
+                bs += NWG;
+                if (bs >= p.nsb) { bs -= p.nsb; bph ^= 1u; }
+                const uint32_t blo = (((bbuf + s * b_slot_bytes) & 0x3FFFFu) >> 4) | (1u << 16);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    if (id0[j] == 0u) continue;
+                    const uint32_t slot = wg * SPW + sl;
+                    if (!ready) mbar_wait_blk(A_FULL(slot), slph);
+                    if (++sl == SPW) { sl = 0; slph ^= 1u; }
+                    ready = mbar_test(A_FULL(wg * SPW + sl), slph);
+                    tc_fence_after();
+                    const uint32_t a_addr = a_tmem + slot * 64;
+                    const uint32_t lo = blo + bo[j];
+#pragma unroll
+                    for (int k = 0; k < GS / 16; ++k)
+                        tc_mma_ts_lohi(dc[j], a_addr + k * 8, lo + (k >> 2) * SLAB_STEP + (k & 3) * 2, DESC_HI, id0[j],
+                                       j == 0 && k == 0 ? accum : 1u);       // the first tile covers every column
+                    tc_commit(A_EMPTY(slot));
+                }
+                accum = 1;
+                tc_commit(B_EMPTY(s));
+            }
+            if (accum) tc_commit(D_FULL(wg));
+            else mbar_arrive(D_FULL(wg));                            // no group of this item was this warpgroup's
+        }
+        // all MMAs must be complete before TMEM is freed
+        if (ic > 0) mbar_wait(D_FULL(wg), (ic - 1) & 1u, abort_flag, p.status, true);
+        }
+        __syncwarp();
+    } else {
+        // ---------------- dequant + epilogue warps: the warpgroups take the K-groups in turn (counted over the items) ----------------
+        const int wg = warp >> 2;
+        const int r = threadIdx.x & 127;         // row of the tile = TMEM lane
+        // lanes 2i and 2i + 1 hold row i of the tile's first and second packed block (mode 0: the gate and the up row of
+        // one hidden unit, which the epilogue pairs with a shuffle)
+        const int blk = r & 1, rr = r >> 1;
+        const uint32_t lane_addr = ((uint32_t)((warp & 3) * 32)) << 16;
+        uint32_t sl = 0, slph = 1, ic = 0;
+        int turn = wg;                                  // groups until this warpgroup's next one
+        uint32_t wph = 0;                               // weight ring: slot and parity advance by addition
+        int ws = wg;
+        for (uint32_t qi = 0;; ++qi, ++ic) {
+            const int item = pop(qi, true);
+            if (item < 0) break;
+            const ItemInfo ii = decode_item(p, item);
+            const TcUnit* u = p.units + ii.unit;
+            const int e = u->e, kmax = u->kmax;
+            const uint8_t* mat = p.mode == 0 ? p.P.w[3 * e + blk] : p.P.w[3 * e + 2];
+            const int S = matrix_exponent(mat, WPACK ? 0 : p.L.seg_shift[0] - (p.L.top - p.L.b1));
+            const float two_mS = exp2f((float)-S);
+            const int smax = p.L.last_seg[kmax];                 // stored segments 0..smax
+            const long long row0 = u->row0;                      // read here: the epilogue must not wait for it
+            const int ncols = u->ncols;
+            int pc0[8], pcn[8], prl[8];                          // per piece: first column, columns, real columns
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+                pc0[kk] = u->col0[kk]; pcn[kk] = kk <= kmax ? u->cnt[kk] : 0; prl[kk] = u->real[kk];
+            }
+            auto nreal_of = [&](int c0) -> int {               // real tokens among the 16 columns from c0
+                int nreal = 0;
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    const int rel = c0 - pc0[kk];
+                    if (pcn[kk] > 0 && rel >= 0 && rel < pcn[kk]) nreal = min(16, max(0, prl[kk] - rel));
+                }
+                return nreal;
+            };
+            auto hand_over = [&](uint32_t slot) {
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(A_FULL(slot));
+                if (++sl == SPW) { sl = 0; slph ^= 1u; }
+            };
+
+            const int turn0 = turn, n_groups = ii.g1 - ii.g0;
+#pragma unroll 1
+            for (int G = ii.g0; G < ii.g1; ++G) {
+                if (turn != 0) { --turn; continue; }                 // another warpgroup's
+                turn = NWG - 1;
+                const int s = ws;
+                mbar_wait_blk(W_FULL(s), wph);
+                ws += NWG;
+                if (ws >= nsw) { ws -= nsw; wph ^= 1u; }
+                const uint32_t wb = wbuf + s * w_slot_bytes + blk * p.L.block_bytes;
+                uint32_t meta;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(meta) : "r"(wb + 4u * rr));
+                const __half2 mh = as_h2(meta);
+                const float s1 = __low2float(mh) * two_mS, lo = __high2float(mh) * two_mS;
+                if constexpr (WPACK != 0) {
+                    using WL = WidthList<WPACK>;
+                    auto step = [&](auto jc) {
+                        constexpr int J = decltype(jc)::value;
+                        if constexpr (J < WL::count()) {
+                            if (J <= kmax) {
+                                constexpr int SW = WL::sw(J), NT = J > 0 ? SW : 1;
+                                constexpr int SC = D2MOE_TILE_ROWS * 2 * (WL::top() - WL::pos(J) - WL::w(0));   // scales of the steps up to here
+                                constexpr int CS = GS * SW / 8 < 16 ? GS * SW / 8 : 16;
+                                const uint32_t slot = wg * SPW + sl;
+                                const bool free_slot = mbar_test(A_EMPTY(slot), slph);      // asked for early: the answer takes a while
+                                SegTile<GS, SW, NT> T;
+                                T.load(wb + (uint32_t)(WL::seg_off(GS, J) + SC) + (uint32_t)(rr * CS));
+                                if constexpr (J == 0) {
+                                    field_mults<SW>(s1 * 16777216.0f, T.mult[0]);
+                                    T.c = as_u32(h2dup(lo));
+                                } else {
+                                    float sum = 0.0f;
+#pragma unroll
+                                    for (int t = 0; t < NT; ++t) {               // bit t's scale lies t planes before that of the lowest bit
+                                        unsigned short raw;
+                                        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(raw)
+                                                     : "r"(wb + (uint32_t)(WL::seg_off(GS, J) + SC - D2MOE_TILE_ROWS * 2 * (1 + t)) + 2u * rr));
+                                        const float sl = __half2float(__ushort_as_half(raw)) * two_mS;
+                                        sum += sl;
+                                        field_mults<SW>(sl * __int_as_float((127 + 25 - t) << 23), T.mult[t]);
+                                    }
+                                    T.c = as_u32(h2dup(-sum));
+                                }
+                                uint32_t v[16];
+                                T.block(0, v);
+                                if (!free_slot) mbar_wait_blk(A_EMPTY(slot), slph);
+                                tc_fence_after();
+                                const uint32_t dst = a_tmem + slot * 64 + lane_addr;
+                                tc_st16(dst, v);
+#pragma unroll
+                                for (int b = 1; b < GS / 32; ++b) {
+                                    uint32_t v2[16];
+                                    T.block(b, v2);
+                                    tc_st16(dst + b * 16, v2);
+                                }
+                                hand_over(slot);
+                            }
+                        }
+                    };
+                    step(std::integral_constant<int, 0>{});
+                    step(std::integral_constant<int, 1>{});
+                    step(std::integral_constant<int, 2>{});
+                    step(std::integral_constant<int, 3>{});
+                } else {
+#pragma unroll 1
+                    for (int sj = 0; sj <= smax; ++sj) {
+                        const int4 tb = seg_tab[sj];
+                        const int sw = tb.x & 255;
+                        const uint32_t seg = wb + (uint32_t)tb.y;
+                        const float M = s1 * __int_as_float(tb.z);
+                        const uint32_t c = sj == 0 ? as_u32(h2dup(lo)) : 0u;
+                        const uint32_t slot = wg * SPW + sl;
+                        mbar_wait_blk(A_EMPTY(slot), slph);
+                        tc_fence_after();
+                        const uint32_t dst = a_tmem + slot * 64 + lane_addr;
+                        auto take = [&](auto swc) {
+                            constexpr int SW = decltype(swc)::value;
+                            constexpr int CS = GS * SW / 8 < 16 ? GS * SW / 8 : 16;
+                            const uint32_t row = seg + (uint32_t)(rr * CS);
+                            if (((tb.x >> 8) & 255) > 0) {
+                                if constexpr (SW < 8) write_bits<GS, SW>(row, wb + (uint32_t)tb.w + 2u * rr, two_mS, dst);
+                            } else {
+                                write_segment<GS, SW>(row, M * 16777216.0f, c, dst);
+                            }
+                        };
+                        if (sw == 1) take(std::integral_constant<int, 1>{});
+                        if (sw == 2) take(std::integral_constant<int, 2>{});
+                        if (sw == 4) take(std::integral_constant<int, 4>{});
+                        if (sw == 8) take(std::integral_constant<int, 8>{});
+                        hand_over(slot);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(W_EMPTY(s));
+            }
+
+            // ---- epilogue: D (128 rows x ncols, the sum of both accumulators) -> global; the warpgroups take 16-column chunks in turn.  SwiGLU is split between the
+            // two threads of a hidden unit (the gate row's thread finishes the first eight tokens of a chunk, the up row's thread the
+            // other eight).  Padding columns (their activation rows and scale factors are never written) are neither stored nor
+            // checked.
+            const float two_S = exp2f((float)S);
+            const int keep = blk == 0 ? 0 : 8;
+            uint32_t overbits = 0;                               // largest |h| seen, as bits (a NaN above every number)
+            // a warpgroup may have had no group of a short item
+            const bool has0 = (wg == 0 ? turn0 : (turn0 ^ 1)) < n_groups, has1 = (wg == 1 ? turn0 : (turn0 ^ 1)) < n_groups;
+            mbar_wait_blk(D_FULL(0), ic & 1);
+            mbar_wait_blk(D_FULL(1), ic & 1);
+            tc_fence_after();
+#pragma unroll 1
+            for (int c0 = wg * 16; c0 < ncols; c0 += 16 * NWG) {
+                const long long grow = row0 + c0;
+                uint32_t va[16], vb[16];
+                tc_ld16(d_tmem + lane_addr + c0, va);
+                tc_ld16(d_tmem + CAP + lane_addr + c0, vb);
+                const int nreal = nreal_of(c0);
+                auto add_accumulators = [&]() {
+                    tc_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        va[j] = __float_as_uint((has0 ? __uint_as_float(va[j]) : 0.0f) + (has1 ? __uint_as_float(vb[j]) : 0.0f));
+                };
+                if (p.mode == 0) {
+                    const float4* xp = reinterpret_cast<const float4*>(p.row_scale + grow + keep);
+                    const float4* hp = reinterpret_cast<const float4*>(p.row_scale + p.R_alloc + grow + keep);
+                    const float4 x0 = xp[0], x1 = xp[1], h0 = hp[0], h1 = hp[1];
+                    const float xs[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                    const float hq[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+                    __half* dst = p.hbuf + (grow + keep) * p.D.F + (long long)ii.tile * 64 + rr;
+                    add_accumulators();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        // (the two rows may belong to matrices of different S: each thread scales its own)
+                        const float other = __shfl_xor_sync(0xffffffffu, __uint_as_float(blk == 0 ? va[8 + j] : va[j]) * two_S, 1) * xs[j];
+                        const float mine = __uint_as_float(blk == 0 ? va[j] : va[8 + j]) * two_S * xs[j];
+                        const float g = blk == 0 ? mine : other, up = blk == 0 ? other : mine;
+                        float h = __fdividef(g, 1.0f + __expf(-g)) * up * hq[j];
+                        if (keep + j < nreal) {
+                            const uint32_t hb = __float_as_uint(h) & 0x7fffffffu;
+                            overbits = max(overbits, hb);
+                            // beyond fp16 even at the token's own scale (or not a number): stored as zero, call flagged below
+                            if (hb > 0x477fe000u) h = 0.0f;                  // bits of 65504
+                            dst[(long long)j * p.D.F] = __float2half_rn(h);
+                        }
+                    }
+                } else {
+                    const float4* a = reinterpret_cast<const float4*>(p.row_scale + 2 * p.R_alloc + grow);
+                    const float4 h0 = a[0], h1 = a[1], h2 = a[2], h3 = a[3];
+                    const float hs[16] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w, h2.x, h2.y, h2.z, h2.w, h3.x, h3.y, h3.z, h3.w};
+                    float* dst = p.obuf + (long long)ii.split * p.R_alloc * p.D.d + grow * p.D.d + (long long)ii.tile * 128 + blk * 64 + rr;
+                    add_accumulators();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j)
+                        if (j < nreal) dst[(long long)j * p.D.d] = __uint_as_float(va[j]) * two_S * hs[j];
+                }
+            }
+            if (p.mode == 0 && overbits > 0x477fe000u && p.status) atomicOr(p.status, D2MOE_DEV_NONFINITE);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) { mbar_arrive(D_EMPTY(0)); mbar_arrive(D_EMPTY(1)); }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == WARP_MMA) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_ffn_step(const d2moe_config* c, const MoeDims& D, const PackLayout& Lgu, const PackLayout& Ld,
+                            const ExpertPtrs& P, const TcPlan& pl, const TcBuffers& B, int32_t* device_status, cudaStream_t st, void* const* ev) {
+    auto mark = [&](int i) { if (ev) cudaEventRecord((cudaEvent_t)ev[i], st); };
+    const int sms = device_sm_count();
+    TmaMaps maps_x, maps_h;
+    if (!make_maps(&maps_x, B.xp16, pl.R_alloc, D.d) || !make_maps(&maps_h, B.h16, pl.R_alloc, D.F))
+        return cudaErrorNotSupported;
+
+    for (int mode = 0; mode < 2; ++mode) {
+        StepParams p;
+        p.D = D; p.L = mode == 0 ? Lgu : Ld; p.P = P; p.mode = mode;
+        p.n_row_tiles = mode == 0 ? D.F / 64 : D.d / 128;
+        p.n_split = mode == 0 ? 1 : pl.n_split;
+        p.groups_per_split = mode == 0 ? p.L.n_groups : pl.groups_per_split;
+        p.units = B.units; p.n_units = B.n_units; p.next_item = B.n_units + 1 + mode;
+        p.hbuf = B.h16; p.obuf = B.o32; p.row_scale = B.slot_f; p.R_alloc = pl.R_alloc; p.status = device_status;
+        p.nsb = pl.n_cap == 64 ? 4 : 3;
+        const int b_bytes = p.nsb * pl.n_cap * D.g * 2;
+        const int w_slot = 2 * p.L.block_bytes;
+        const int bar_bytes = 1024;
+        const int budget = 226 * 1024;
+        int nsw = (budget - b_bytes - bar_bytes - 512 - 1024) / w_slot;
+        if (nsw > MAX_NSW) nsw = MAX_NSW;
+        if (nsw < NWG) return cudaErrorInvalidConfiguration;
+        p.nsw = nsw;
+        p.smem_w_off = b_bytes;
+        p.smem_bar_off = (b_bytes + nsw * w_slot + 511) & ~511;     // 512-byte aligned from the 1024-byte aligned base
+        const int smem_bytes = p.smem_bar_off + bar_bytes + 1024;   // + slack for the 1024-byte alignment
+        mark(mode == 0 ? 1 : 2);
+        // lists of at most four steps that are one stored segment each (nibble j = width of step j)
+        int wpack = 0;
+        if (p.L.n_seg <= 4 && p.L.n_seg == p.L.n_widths)
+            for (int j = 0; j < p.L.n_seg; ++j) wpack |= p.L.seg_w[j] << (4 * j);
+        auto launch = [&](auto kc) -> cudaError_t {
+            constexpr auto kern = decltype(kc)::value;
+            cudaError_t err = ensure_dynamic_smem<kern>(smem_bytes);
+            if (err != cudaSuccess) return err;
+            launch_chained(kern, dim3(sms), dim3(ST_THREADS), smem_bytes, st, p, mode == 0 ? maps_x : maps_h);
+            return cudaSuccess;
+        };
+#define ST_KERNEL(GS_, WP_, CAP_) std::integral_constant<decltype(&ffn_step_kernel<GS_, WP_, CAP_>), &ffn_step_kernel<GS_, WP_, CAP_>>{}
+#define ST_LAUNCH(GS_, WP_) (pl.n_cap == 64 ? launch(ST_KERNEL(GS_, WP_, 64)) : launch(ST_KERNEL(GS_, WP_, 128)))
+        cudaError_t e;
+        if (D.g == 128 && wpack == 0x4112) e = ST_LAUNCH(128, 0x4112);        // {2,3,4,8}
+        else if (D.g == 128 && wpack == 0x422) e = ST_LAUNCH(128, 0x422);     // {2,4,8}
+        else if (D.g == 128) e = ST_LAUNCH(128, 0);
+        else e = ST_LAUNCH(64, 0);
+#undef ST_LAUNCH
+#undef ST_KERNEL
+        if (e != cudaSuccess) return e;
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}

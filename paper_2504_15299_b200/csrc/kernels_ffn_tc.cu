@@ -971,7 +971,7 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
     // (the 8-bit kernel folds one scale per group into its integer accumulators, which needs the tied residual
     // scales: with free scales every load takes the grouped GEMM)
     pl->decode = (avg <= D2MOE_DECODE_MAX_AVG && c->scale_mode == 0) ? 1 : 0;
-    pl->rows = 0;
+    pl->rows = pl->step = 0;
     if (pl->decode) {
         pl->n_cap = 32;                      // token slots per unit
     } else {
@@ -988,7 +988,14 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
         // 96; Mixtral shape 150: 1012 / 1066, 160: 1115 / 1077; 16 experts of F 1408: 142: 134 / 136, 154: 144 / 138).
         const bool straight = c->group_size == 128 && c->n_bits == 4 && c->bits[0] == 2 && c->bits[1] == 3 && c->bits[2] == 4 && c->bits[3] == 8;
         pl->n_cap = avg <= 96 ? 128 : (avg <= (straight ? 152 : 160) && c->scale_mode == 0 ? 192 : 320);
-        pl->rows = pl->n_cap <= 192 ? 1 : 0;
+        // Free scales, decode-sized loads: a tile per segment (ffn_step_kernel).  Up to three tokens an expert most units hold one width or
+        // two, which the running sum serves with as many tiles: with short rows, where an item's start and end weigh more, that is
+        // the faster one (64 experts of F 1408, 16 tokens: 295 us, this way 302, 22: 303 / 308, 48: 407 / 385; 8 experts of F 14336, 1 token: 135 / 118).
+        // Units of 64 columns where an expert's tokens and the padding of its pieces (8 columns on average) leave room in them:
+        // Mixtral shape, 25 tokens per expert 796 us with units of 128, 738 with 64.
+        pl->step = c->scale_mode == 1 && avg <= D2MOE_DECODE_MAX_AVG && (avg > 3 || c->d_ffn / c->group_size >= 32) ? 1 : 0;
+        if (pl->step && avg + 8 * c->n_bits <= 57) pl->n_cap = 64;
+        pl->rows = pl->n_cap <= 192 && !pl->step ? 1 : 0;
     }
     const long long n_pieces = pl->decode ? (long long)c->n_experts + c->n_shared
                                           : (long long)c->n_experts * c->n_bits + c->n_shared;
@@ -998,13 +1005,15 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl) {
                                     : A_tot + 15 * (n_pieces < A_tot ? n_pieces : A_tot);
     pl->pad_rows = pad_rows;
     pl->R_alloc = ((pad_rows + 255) / 256) * 256 + 256;
-    // (grouped GEMM: as if every unit held 128 columns, so that the unit list never shrinks when T grows)
-    pl->max_units = (int)(c->n_experts + c->n_shared + pl->R_alloc / (pl->decode ? pl->n_cap : 128) + 1);
+    // (grouped GEMM: as if every unit held 64 columns, so that the unit list never shrinks when T grows)
+    pl->max_units = (int)(c->n_experts + c->n_shared + pl->R_alloc / (pl->decode ? pl->n_cap : 64) + 1);
     // split-K of the down projection: aim for >= 4 work items per resident CTA
-    long long units_est = (c->n_experts < A ? c->n_experts : A) + (long long)c->n_shared * ((T + pl->n_cap - 1) / pl->n_cap);
+    // (units of 64 are counted as units of 128: the split has to fall as T grows)
+    const int cap = pl->n_cap == 64 ? 128 : pl->n_cap;
+    long long units_est = (c->n_experts < A ? c->n_experts : A) + (long long)c->n_shared * ((T + cap - 1) / cap);
     // prefill-sized loads: an expert spans several units (every partial output plane is written by the down
     // projection and read again by the combine, so no more planes than the work distribution needs)
-    if (!pl->decode && units_est < A / pl->n_cap + c->n_experts / 2) units_est = A / pl->n_cap + c->n_experts / 2;
+    if (!pl->decode && units_est < A / cap + c->n_experts / 2) units_est = A / cap + c->n_experts / 2;
     const long long tiles = c->d_model / 128;
     const int n_groups = c->d_ffn / c->group_size;
     const long long ctas = pl->decode ? 296 : 148;       // resident CTAs: 2 per SM (decode kernel), 1 per SM
@@ -1038,6 +1047,7 @@ cudaError_t launch_ffn_tensor(const d2moe_config* c, const MoeDims& D, const Pac
                    pl.max_units, sms, device_status);
     launch_chained(tc_gather_kernel, dim3((unsigned)(pl.pad_rows < 16 * sms ? pl.pad_rows : 16 * sms)), dim3(128), 0, st, D.d, x, B.src_token, B.pad_off, n_keys, B.xp16, B.slot_f, pl.R_alloc, device_status);
 
+    if (pl.step) return launch_ffn_step(c, D, Lgu, Ld, P, pl, B, device_status, st, ev);
     if (pl.rows) return launch_ffn_row(c, D, Lgu, Ld, P, pl, B, device_status, st, ev);
 
     TmaMaps maps_x, maps_h;

@@ -32,6 +32,7 @@ struct I8Unit {
 struct TcPlan {
     int decode;             // 1: memory-bound 8-bit decode kernel (tokens laid out widest first, scales applied
                             //    to the accumulators); 0: grouped fp16 dequant-GEMM (one tile per width, any load)
+    int step;               // 1: grouped GEMM with one operand tile per stored segment (free scales, decode-sized loads)
     int rows;               // 1: grouped GEMM with whole rows per thread (small units), 0: with half rows (large units)
     int n_cap;              // columns per unit
     long long pad_rows;     // most padded rows any routing of the call can give
@@ -60,6 +61,8 @@ void tc_plan(const d2moe_config* c, long long T, TcPlan* pl);
 cudaError_t launch_ffn_tensor(const d2moe_config* c, const MoeDims& D, const PackLayout& Lgu, const PackLayout& Ld,
                               const ExpertPtrs& P, const __nv_bfloat16* x, const RouteBufs& R, const TcPlan& pl,
                               const TcBuffers& B, int32_t* device_status, cudaStream_t st, void* const* ev, bool supplied);
+cudaError_t launch_ffn_step(const d2moe_config* c, const MoeDims& D, const PackLayout& Lgu, const PackLayout& Ld,
+                            const ExpertPtrs& P, const TcPlan& pl, const TcBuffers& B, int32_t* device_status, cudaStream_t st, void* const* ev);
 cudaError_t launch_ffn_row(const d2moe_config* c, const MoeDims& D, const PackLayout& Lgu, const PackLayout& Ld,
                            const ExpertPtrs& P, const TcPlan& pl, const TcBuffers& B, int32_t* device_status, cudaStream_t st, void* const* ev);
 // group_keys: when not null, the sort keys of the assignments whose grouping (group_off, perm, inv_perm of R) is
