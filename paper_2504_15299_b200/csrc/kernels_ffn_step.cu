@@ -1,6 +1,7 @@
-// Grouped dequant-GEMM on the 5th-generation tensor cores for decode-sized loads with free residual scales: one operand tile per
-// stored segment.
+// Grouped dequant-GEMM on the 5th-generation tensor cores with an issuer and an accumulator per dequant warpgroup: decode-sized
+// loads with free residual scales (one operand tile per stored segment) and small units with tied scales (TIED).
 //
+// Free scales.
 // The nested code is a sum over its segments (W_hat at a width = the base's share + the shares of the steps up to that width), and a
 // product with a sum is a sum of products: the tile of a segment holds that segment's share alone (base: lo + s1 Q; a step of w bits:
 // sum over its bits of s_l (2 bit_l - 1), its constant in the first addend) and is multiplied by the tokens of its width and of all wider
@@ -9,6 +10,14 @@
 // registers at a time), and a share is rounded at its own magnitude instead of the weight's: the error of a layer call against 64
 // bits falls from 1.768e-3 to 1.679e-3 (d 4096, F 14336, {2,3,4,8}, 64 tokens; no list measured worse).  It costs products, the sum of the suffixes instead of
 // the columns once, which is little while a unit holds few tokens.
+//
+// Tied scales, width lists known at compile time.  Units hold up to 192 tokens, and a product for every suffix would keep the tensor
+// cores busy for longer than the dequantization takes.  So the running tile goes up to the second widest width (whose constant is in
+// the first addend: its tile goes out as it is; narrower widths get the difference in an addition), and the tokens of the widest
+// width are multiplied by that tile and by one more with the share of the last step alone.  Against ffn_row_kernel that is 64
+// additions a row less, no loop over stored segments, and the products of the widest tokens twice; error against 64 bits
+// 2.203e-3 -> 2.115e-3 (333 tokens; {2,4,8} 2.197 -> 2.115).  Units of 128 leave two tiles a warpgroup, units of 192 one.
+// The same straight-line dequantization with one issuer in group order took 1003 us where this takes 683.
 //
 // The two dequant warpgroups take alternate K-groups, whole rows per thread, and share nothing: each has operand tiles, an issuing
 // thread and an accumulator of its own, and the epilogue adds the two accumulators.  With one issuer in group order a warpgroup
@@ -20,7 +29,8 @@
 // What bounds it: the dependent arithmetic of two dequant warps per scheduler (about 3.3 cycles an instruction; 1050 instructions per row
 // and group, 896 of them the AND and the packed FMA of seven steps).  Measured (layer call, ffn_row_kernel -> this kernel): d 4096, F
 // 14336, 8 experts, top-2, {2,3,4,8}: 1 token 135 -> 118 us, 8 579 -> 485, 64 1020 -> 740, 160 1057 -> 830; {2,4,8} 64 tokens 920 ->
-// 696; {5,6,7,8} 945 -> 872; 64 experts of F 1408, top-6, 256 tokens 519 -> 439.
+// 696; {5,6,7,8} 945 -> 872; 64 experts of F 1408, top-6, 256 tokens 519 -> 439.  Tied: Mixtral shape, {2,3,4,8}: 180 tokens 807 -> 655,
+// 333 830 -> 683, 440 916 -> 792, 600 988 -> 901; {2,4,8} 333 tokens 667 -> 557; 64 experts of F 1408, 512 tokens 431 -> 387.
 //
 // Warp roles (384 threads, 1 CTA per SM, all 512 TMEM columns): warps 0-3 and 4-7 the dequant warpgroups (thread = weight row =
 // TMEM lane; lanes 2i and 2i + 1 hold row i of the tile's two packed blocks, for gate/up the two rows of one hidden unit, which the
@@ -41,7 +51,7 @@ constexpr int WARP_WPROD = 4 * NWG, WARP_BPROD = WARP_WPROD + 1, WARP_MMA = WARP
 constexpr int TMEM_COLS = 512;
 constexpr int MAX_SPW = 3;
 // operand tiles (64 TMEM columns each, behind the accumulators) per warpgroup, for accumulators of CAP columns
-__host__ __device__ constexpr int tiles_per_wg(int cap) { return cap <= 64 ? 3 : 2; }
+__host__ __device__ constexpr int tiles_per_wg(int cap) { return cap <= 64 ? 3 : (cap <= 128 ? 2 : 1); }
 constexpr int MAX_NSB = 4;             // activation ring depth (upper bound)
 constexpr int MAX_NSW = 8;             // weight ring depth (upper bound)
 constexpr int NSQ = 4;                 // entries of the work queue between the weight producer and the other warps
@@ -188,12 +198,16 @@ __device__ __forceinline__ ItemInfo decode_item(const StepParams& p, int item) {
     return it;
 }
 
-// WPACK: a width list whose steps are one stored segment each (nibble j: width of step j), 0: any list; CAP: columns of a unit
-template <int GS, int WPACK, int CAP>
+// WPACK: a width list whose steps are one stored segment each (nibble j: width of step j), 0: any list; CAP: columns of a unit;
+// TIED: scale_mode 0
+template <int GS, int WPACK, int CAP, bool TIED>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ TmaMaps maps) {
     constexpr int HALVES = GS / 64;              // 64-element K slabs of the activation tile
     constexpr int SPW = tiles_per_wg(CAP);
+    constexpr int KW = WidthList<WPACK>::count();   // widths of a list known at compile time
+    constexpr int TILE_COLS = GS / 2;            // TMEM columns of one operand tile
+    static_assert(!TIED || (KW >= 3 && TILE_COLS == 64), "tied scales: lists known at compile time");
     static_assert(NWG == 2 && SPW <= MAX_SPW && NWG * (CAP + 64 * SPW) <= 512, "tensor memory");
     extern __shared__ uint8_t smem_raw[];
     // shared layout (from a 1024-byte boundary, which the 128B-swizzled operand tiles need):
@@ -379,6 +393,18 @@ ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ Tm
             uint32_t id0[8], dc[8], bo[8];                        // per stored segment: descriptor, D column, B rows / 16 B
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
+                if constexpr (TIED) {
+                    // up to the second widest width a tile per width, that one also for the widest tokens, which have the last one besides
+                    int cnt = j <= kmax ? u->cnt[j] : 0, col0 = u->col0[j];
+                    if (j == KW - 2 && j <= kmax) {
+                        if (cnt == 0) col0 = u->col0[KW - 1];
+                        cnt = ncols - col0;
+                    }
+                    id0[j] = cnt ? instr_desc_f16(cnt) : 0u;
+                    dc[j] = d_tmem + wg * CAP + col0;
+                    bo[j] = (uint32_t)col0 * 8u;
+                    continue;
+                }
                 // its tile is multiplied by the tokens of its width and of the wider ones
                 int col0 = ncols;
                 if (j < p.L.n_seg) for (int kk = kmax; kk >= p.L.seg_kk[j]; --kk) col0 = u->cnt[kk] > 0 ? u->col0[kk] : col0;
@@ -410,7 +436,7 @@ ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ Tm
 #pragma unroll
                     for (int k = 0; k < GS / 16; ++k)
                         tc_mma_ts_lohi(dc[j], a_addr + k * 8, lo + (k >> 2) * SLAB_STEP + (k & 3) * 2, DESC_HI, id0[j],
-                                       j == 0 && k == 0 ? accum : 1u);       // the first tile covers every column
+                                       k == 0 && (TIED ? j != KW - 1 : j == 0) ? accum : 1u);   // the first tile of a column
                     tc_commit(A_EMPTY(slot));
                 }
                 accum = 1;
@@ -445,6 +471,8 @@ ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ Tm
             const int S = matrix_exponent(mat, WPACK ? 0 : p.L.seg_shift[0] - (p.L.top - p.L.b1));
             const float two_mS = exp2f((float)-S);
             const int smax = p.L.last_seg[kmax];                 // stored segments 0..smax
+            unsigned present = 0;
+            for (int kk = 0; kk <= kmax; ++kk) present |= (u->cnt[kk] > 0 ? 1u : 0u) << kk;
             const long long row0 = u->row0;                      // read here: the epilogue must not wait for it
             const int ncols = u->ncols;
             int pc0[8], pcn[8], prl[8];                          // per piece: first column, columns, real columns
@@ -483,7 +511,84 @@ ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ Tm
                 asm volatile("ld.shared.u32 %0, [%1];" : "=r"(meta) : "r"(wb + 4u * rr));
                 const __half2 mh = as_h2(meta);
                 const float s1 = __low2float(mh) * two_mS, lo = __high2float(mh) * two_mS;
-                if constexpr (WPACK != 0) {
+                if constexpr (TIED) {
+                    uint32_t acc[GS / 2];                                // the running tile
+                    // A list known at compile time (at least three widths).  The running tile goes up to the second widest width, whose
+                    // constant is in the first addend; narrower widths get the difference.  Tokens of the widest width are
+                    // multiplied by that tile too and by one more, the share of the last step alone, which needs no running tile and no
+                    // addition.
+                    using WL = WidthList<WPACK>;
+                    const float c_wide = 0.5f * s1 * pow2i(-(WL::bits(KW - 2) - WL::w(0)));
+                    uint32_t free_slot = 0, slot = 0;
+                    auto look_ahead = [&]() {                            // (asked for early: the answer takes a while)
+                        slot = wg * SPW + sl;
+                        free_slot = mbar_test(A_EMPTY(slot), slph);
+                    };
+                    auto acquire = [&]() -> uint32_t {
+                        if (!free_slot) mbar_wait_blk(A_EMPTY(slot), slph);
+                        __syncwarp();
+                        tc_fence_after();
+                        return a_tmem + slot * 64 + lane_addr;
+                    };
+                    auto step = [&](auto jc) {
+                        constexpr int J = decltype(jc)::value;
+                        if constexpr (J < KW) {
+                            if (J <= kmax) {
+                                constexpr int SW = WL::sw(J), DB = WL::bits(J) - WL::w(0);
+                                constexpr int CS = GS * SW / 8 < 16 ? GS * SW / 8 : 16;
+                                const uint32_t row = wb + (uint32_t)(WL::seg_off(GS, J) + rr * CS);
+                                uint32_t w[GS / 32][SW], mult[8 / SW];
+                                look_ahead();
+#pragma unroll
+                                for (int b = 0; b < GS / 32; ++b) load_block<GS, SW>(row, b, w[b]);
+                                const float M = s1 * pow2i(-DB);
+                                field_mults<SW>(M * 16777216.0f, mult);
+                                constexpr uint32_t FIELD = ((1u << SW) - 1u) * 0x00010001u;
+                                if constexpr (J == KW - 1) {
+                                    const uint32_t c = as_u32(h2dup(0.5f * M - c_wide));
+                                    uint32_t v[16];
+                                    fma_block<SW>(w[0], FIELD, mult, c, v);
+                                    const uint32_t dst = acquire();
+                                    tc_st16(dst, v);
+#pragma unroll
+                                    for (int b = 1; b < GS / 32; ++b) {
+                                        uint32_t v2[16];
+                                        fma_block<SW>(w[b], FIELD, mult, c, v2);
+                                        tc_st16(dst + b * 16, v2);
+                                    }
+                                    hand_over(slot);
+                                } else {
+                                    const uint32_t c = as_u32(h2dup(lo - 0.5f * s1 + c_wide));
+#pragma unroll
+                                    for (int b = 0; b < GS / 32; ++b) {
+                                        uint32_t (&blk16)[16] = *reinterpret_cast<uint32_t (*)[16]>(acc + b * 16);
+                                        if constexpr (J == 0) fma_block<SW>(w[b], FIELD, mult, c, blk16);
+                                        else fma_block_more<SW>(w[b], FIELD, mult, blk16);
+                                    }
+                                    if (J == KW - 2 || ((present >> J) & 1u)) {
+                                        const uint32_t dst = acquire();
+                                        const uint32_t a = as_u32(h2dup(0.5f * M - c_wide));
+#pragma unroll
+                                        for (int b = 0; b < GS / 32; ++b) {
+                                            if constexpr (J == KW - 2) tc_st16(dst + b * 16, *reinterpret_cast<uint32_t (*)[16]>(acc + b * 16));
+                                            else {
+                                                uint32_t v[16];
+#pragma unroll
+                                                for (int i = 0; i < 16; ++i) v[i] = hadd2_bits(acc[b * 16 + i], a);
+                                                tc_st16(dst + b * 16, v);
+                                            }
+                                        }
+                                        hand_over(slot);
+                                    }
+                                }
+                            }
+                        }
+                    };
+                    step(std::integral_constant<int, 0>{});
+                    step(std::integral_constant<int, 1>{});
+                    step(std::integral_constant<int, 2>{});
+                    step(std::integral_constant<int, 3>{});
+                } else if constexpr (WPACK != 0) {
                     using WL = WidthList<WPACK>;
                     auto step = [&](auto jc) {
                         constexpr int J = decltype(jc)::value;
@@ -515,6 +620,7 @@ ffn_step_kernel(const __grid_constant__ StepParams p, const __grid_constant__ Tm
                                 uint32_t v[16];
                                 T.block(0, v);
                                 if (!free_slot) mbar_wait_blk(A_EMPTY(slot), slph);
+                                __syncwarp();
                                 tc_fence_after();
                                 const uint32_t dst = a_tmem + slot * 64 + lane_addr;
                                 tc_st16(dst, v);
@@ -681,10 +787,15 @@ cudaError_t launch_ffn_step(const d2moe_config* c, const MoeDims& D, const PackL
             launch_chained(kern, dim3(sms), dim3(ST_THREADS), smem_bytes, st, p, mode == 0 ? maps_x : maps_h);
             return cudaSuccess;
         };
-#define ST_KERNEL(GS_, WP_, CAP_) std::integral_constant<decltype(&ffn_step_kernel<GS_, WP_, CAP_>), &ffn_step_kernel<GS_, WP_, CAP_>>{}
-#define ST_LAUNCH(GS_, WP_) (pl.n_cap == 64 ? launch(ST_KERNEL(GS_, WP_, 64)) : launch(ST_KERNEL(GS_, WP_, 128)))
+#define ST_KERNEL(GS_, WP_, CAP_, TIED_) std::integral_constant<decltype(&ffn_step_kernel<GS_, WP_, CAP_, TIED_>), &ffn_step_kernel<GS_, WP_, CAP_, TIED_>>{}
+#define ST_LAUNCH(GS_, WP_) (pl.n_cap == 64 ? launch(ST_KERNEL(GS_, WP_, 64, false)) : launch(ST_KERNEL(GS_, WP_, 128, false)))
         cudaError_t e;
-        if (D.g == 128 && wpack == 0x4112) e = ST_LAUNCH(128, 0x4112);        // {2,3,4,8}
+        const bool tied = p.L.scale_mode == 0;
+        if (tied && wpack != 0x4112 && wpack != 0x422) return cudaErrorInvalidConfiguration;      // (tc_plan)
+        if (tied && D.g != 128) return cudaErrorInvalidConfiguration;
+        if (tied && pl.n_cap == 128) e = wpack == 0x4112 ? launch(ST_KERNEL(128, 0x4112, 128, true)) : launch(ST_KERNEL(128, 0x422, 128, true));
+        else if (tied) e = wpack == 0x4112 ? launch(ST_KERNEL(128, 0x4112, 192, true)) : launch(ST_KERNEL(128, 0x422, 192, true));
+        else if (D.g == 128 && wpack == 0x4112) e = ST_LAUNCH(128, 0x4112);        // {2,3,4,8}
         else if (D.g == 128 && wpack == 0x422) e = ST_LAUNCH(128, 0x422);     // {2,4,8}
         else if (D.g == 128) e = ST_LAUNCH(128, 0);
         else e = ST_LAUNCH(64, 0);

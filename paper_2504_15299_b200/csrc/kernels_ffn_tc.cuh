@@ -32,7 +32,8 @@ struct I8Unit {
 struct TcPlan {
     int decode;             // 1: memory-bound 8-bit decode kernel (tokens laid out widest first, scales applied
                             //    to the accumulators); 0: grouped fp16 dequant-GEMM (one tile per width, any load)
-    int step;               // 1: grouped GEMM with one operand tile per stored segment (free scales, decode-sized loads)
+    int step;               // 1: grouped GEMM with an issuer and an accumulator per dequant warpgroup (free scales: decode-sized
+                            //    loads; tied scales: small units of the lists it knows)
     int rows;               // 1: grouped GEMM with whole rows per thread (small units), 0: with half rows (large units)
     int n_cap;              // columns per unit
     long long pad_rows;     // most padded rows any routing of the call can give

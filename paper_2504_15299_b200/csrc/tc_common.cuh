@@ -216,6 +216,8 @@ __device__ __forceinline__ uint32_t hfma2_bits(uint32_t a, uint32_t b, uint32_t 
     asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
     return d;
 }
+// 2^e as a float, -126 <= e <= 127
+__device__ __forceinline__ float pow2i(int e) { return __int_as_float((127 + e) << 23); }
 __device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -242,6 +244,7 @@ struct WidthList {
     __host__ __device__ static constexpr int sw(int j) { return w(j) <= 1 ? 1 : (w(j) <= 2 ? 2 : (w(j) <= 4 ? 4 : 8)); }
     __host__ __device__ static constexpr int count() { int k = 0; while (k < 8 && w(k) != 0) ++k; return k; }
     __host__ __device__ static constexpr int top() { int b = 0; for (int i = 0; i < count(); ++i) b += w(i); return b; }
+    __host__ __device__ static constexpr int bits(int j) { int b = 0; for (int i = 0; i <= j; ++i) b += w(i); return b; }
     __host__ __device__ static constexpr int pos(int j) { int b = 0; for (int i = 0; i <= j; ++i) b += w(i); return top() - b; }
     // a step of w bits is stored as power-of-two fields that add up to exactly w bits per code
     __host__ __device__ static constexpr int seg_off(int gs, int j) { int o = D2MOE_TILE_ROWS * 4; for (int i = 0; i < j; ++i) o += D2MOE_TILE_ROWS * gs * w(i) / 8; return o; }

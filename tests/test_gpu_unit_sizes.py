@@ -68,6 +68,31 @@ def test_free_scales_one_tile_per_segment(B, bits, d, F, g, n_shared):
         assert err <= 1e-2, (T, err)
 
 
+@pytest.mark.parametrize("d,F,n_shared", [(128, 128, 0), (256, 384, 1), (1024, 4096, 0)])
+@pytest.mark.parametrize("bits", [(2, 3, 4, 8), (2, 4, 8)])
+def test_tied_scales_with_an_accumulator_per_warpgroup(B, bits, d, F, n_shared):
+    # The lists known at compile time in units of 128 and 192 columns: every subset of present widths that changes the tiles (the widest
+    # or the second widest missing, one width only), an expert that outgrows its unit, items of one K-group.  Bound as above.
+    E, k, g = 4, 2, 128
+    cfg_tc, cfg_cc = (B.Config(d, F, E, k, g, bits, n_shared=n_shared, kernel_path=p) for p in (0, 1))
+    blobs = [B.pack_mwq(cfg_tc, synth.normal(39, 3 * e + m, (F, d) if m < 2 else (d, F), 0.02, "cuda"))
+             for e in range(E + n_shared) for m in range(3)]
+    K = len(bits)
+    mixes = [[1.0 / K] * K, [0.0] * (K - 1) + [1.0], [0.0] * (K - 2) + [1.0, 0.0], [1.0] + [0.0] * (K - 1), [0.5] + [0.0] * (K - 2) + [0.5]]
+    for T, mix in [(82, 0), (192, 0), (194, 0), (300, 0), (100, 1), (220, 1), (100, 2), (220, 3), (100, 4), (220, 4)]:
+        x = synth.bf16_exact(synth.normal(39, 1000 + T, (T, d), 1.0, "cuda"))
+        logits = synth.normal(39, 2000 + T, (T, E), 1.0, "cuda") + torch.tensor([50.0, 0, 0, -2.5], device="cuda")
+        fb = synth.categorical(39, 3000 + T, (T, k), mixes[mix], "cuda")
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        y1, y1b = (B.moe_forward(cfg_tc, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st) for _ in range(2))
+        y2 = B.moe_forward(cfg_cc, x, blobs, logits=logits, forced_bit_idx=fb, device_status=st).float()
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        assert torch.equal(y1.view(torch.int16), y1b.view(torch.int16)), ("rerun differs", T, mix)
+        err = float(((y1.float() - y2).abs().amax(dim=1) / y2.abs().amax(dim=1)).max())
+        assert err <= 1e-2, (T, mix, err)
+
+
 @pytest.mark.parametrize("scale_mode", [0, 1])
 @pytest.mark.parametrize("bits", [(3, 8), (3, 4, 8), (3, 7), (3, 7, 8), (3, 5), (5, 6, 7, 8)])
 def test_base_width_stored_as_two_fields(B, bits, scale_mode):
