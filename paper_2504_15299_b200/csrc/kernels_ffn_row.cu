@@ -1,4 +1,5 @@
-// Grouped dequant-GEMM on the 5th-generation tensor cores for small units: up to 192 tokens of one expert per work item.
+// Grouped dequant-GEMM on the 5th-generation tensor cores for small units: up to 192 tokens of one expert per work item (the loads
+// that ffn_step_kernel does not take: see tc_plan).
 //
 // The work items, the nested code and its arithmetic (each width's tile built in registers from the one below, one AND and
 // one packed half-precision FMA per code pair), the item queue and the epilogue are those of ffn_tc_kernel.  With few
